@@ -1,7 +1,7 @@
 """Build libdg.so (the C-ABI library) in-tree with nvcc for sm_103a.
 
-The four translation units compile in parallel and link into
-paper_2511_08020_gb300/_lib/libdg.so.  The FP64 throughput probes of the
+The translation units compile in parallel (the element kernels per number of
+points per direction and part) and link into paper_2511_08020_gb300/_lib/libdg.so.  The FP64 throughput probes of the
 benchmark (fp64_probe.cu) link into a library of their own,
 _lib/libfp64probe.so, so that libdg.so carries only the hot path.  Nothing is
 installed elsewhere.
@@ -19,7 +19,10 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIBDIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(LIBDIR, "libdg.so")
-SOURCES = ["dg_host.cpp", "dg_kernels.cu", "dg_moving.cu", "dg_api.cu"]
+SOURCES = ["dg_host.cpp", "dg_kernels.cu", "dg_faces.cu", "dg_moving.cu", "dg_api.cu"]
+# one build per number of points per direction (DG_N = N + 1) and part, the slow ones first
+ELEMENT_SRC = "dg_element.cu"
+ELEMENT_BUILDS = [(n, p) for n in (7, 6, 5, 4, 3, 2) for p in (1, 2, 0)]
 PROBE_SRC = "fp64_probe.cu"
 PROBE_LIB = os.path.join(LIBDIR, "libfp64probe.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
@@ -33,8 +36,8 @@ def nvcc() -> str:
     return path
 
 
-def _compile(src: str, obj: str) -> None:
-    cmd = [nvcc(), *ARCH, *FLAGS, "-c", os.path.join(CSRC, src), "-o", obj]
+def _compile(src: str, obj: str, defines: tuple = ()) -> None:
+    cmd = [nvcc(), *ARCH, *FLAGS, *defines, "-c", os.path.join(CSRC, src), "-o", obj]
     if src.endswith(".cpp"):
         cmd = [nvcc(), *FLAGS, "-x", "c++", "-c", os.path.join(CSRC, src), "-o", obj]
     r = subprocess.run(cmd, capture_output=True, text=True)
@@ -65,9 +68,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
         lib_t = os.path.getmtime(LIB)
         if all(os.path.getmtime(s) <= lib_t for s in srcs):
             return LIB
-    objs = [os.path.join(LIBDIR, os.path.splitext(s)[0] + ".o") for s in SOURCES]
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
-        list(ex.map(_compile, SOURCES, objs))
+    jobs = [(ELEMENT_SRC, f"dg_element_{n}_{p}", (f"-DDG_N={n}", f"-DDG_PART={p}")) for n, p in ELEMENT_BUILDS]
+    jobs += [(s, os.path.splitext(s)[0], ()) for s in SOURCES]
+    objs = [os.path.join(LIBDIR, name + ".o") for _, name, _ in jobs]
+    with cf.ThreadPoolExecutor(max_workers=len(jobs)) as ex:
+        list(ex.map(_compile, [j[0] for j in jobs], objs, [j[2] for j in jobs]))
     tmp = LIB + ".tmp"
     cmd = [nvcc(), *ARCH, "-shared", "-cudart", "shared", "-o", tmp, *objs]
     r = subprocess.run(cmd, capture_output=True, text=True)

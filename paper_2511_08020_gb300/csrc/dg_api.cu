@@ -148,6 +148,7 @@ struct dg_mesh {
   // device data
   double* d_dpool = nullptr;
   int* d_ipool = nullptr;
+  dgk::FixPair* d_fpool = nullptr;
   dgk::TypeTab* d_tabs = nullptr;
   int* d_slot_tab = nullptr;
   int8_t* d_slot_type = nullptr;
@@ -355,6 +356,7 @@ struct dg_mesh {
     dgk::Ctx c;
     c.dpool = d_dpool;
     c.ipool = d_ipool;
+    c.fpool = reinterpret_cast<const int2*>(d_fpool);
     c.tabs = d_tabs;
     c.slot_tab = d_slot_tab;
     c.slot_type = d_slot_type;
@@ -393,6 +395,8 @@ struct dg_mesh {
     c.flux = flux;
     c.split = split;
     c.nQmax = nQmax;
+    c.nmask = 0u;
+    for (const auto& T : h.tables.tabs) c.nmask |= 1u << T.n;
     if (moving) {
       c.mpool = d_mpool;
       c.slot_moff = d_slot_moff;
@@ -738,6 +742,7 @@ struct dg_mesh {
         for (const auto& G : groups) {
           dgk::Ctx cg = c;
           cg.nQmax = G.n * G.n * G.n;
+          cg.nmask = 1u << G.n;
           dgk::Sched s{G.d_list, G.nchunks, G.d_chunks, d_counters + parity, d_counters + (parity ^ 1)};
           dgk::launch_element(cg, mode, a, s, true, num_sms * (mode == dgk::kNsVolume ? G.bpsm_ns : G.bpsm), G.wpb,
                               st);
@@ -745,10 +750,15 @@ struct dg_mesh {
         }
       } else if ((scheduler == DG_SCHED_STATIC || scheduler == DG_SCHED_WEIGHTED) && !per_elem) {
         const bool wt = scheduler == DG_SCHED_WEIGHTED;
-        dgk::Sched s{nullptr, wt ? nchunks_weighted : nchunks_static, wt ? d_chunks_weighted : d_chunks_static,
-                     d_counters + parity, d_counters + (parity ^ 1)};
-        dgk::launch_element(c, mode, a, s, true, mode == dgk::kNsVolume ? grid_ns() : grid_balanced(), wpb, st);
-        parity ^= 1;
+        for (int n = 2; n <= dgk::kMaxn; ++n) {   // one launch per degree present
+          if (!((c.nmask >> n) & 1u)) continue;
+          dgk::Ctx cg = c;
+          cg.nmask = 1u << n;
+          dgk::Sched s{nullptr, wt ? nchunks_weighted : nchunks_static, wt ? d_chunks_weighted : d_chunks_static,
+                       d_counters + parity, d_counters + (parity ^ 1)};
+          dgk::launch_element(cg, mode, a, s, true, mode == dgk::kNsVolume ? grid_ns() : grid_balanced(), wpb, st);
+          parity ^= 1;
+        }
       } else {
         for (int t = 0; t < 4; ++t) {
           if (h.type_slots[t].empty()) continue;
@@ -918,7 +928,7 @@ struct dg_mesh {
   }
 
   void release() {
-    void* ptrs[] = {d_dpool, d_ipool, d_tabs, d_slot_tab, d_slot_type, d_slot_qoff, d_slot_hoff, d_slot_ftoff,
+    void* ptrs[] = {d_dpool, d_ipool, d_fpool, d_tabs, d_slot_tab, d_slot_type, d_slot_qoff, d_slot_hoff, d_slot_ftoff,
                     d_elem_of_slot, d_elem_qoff, d_elem_voff, d_geo, d_H, d_T, d_faces, d_fblocks, d_perms, d_dense, d_status,
                     d_cost, d_smns, d_counters, d_chunks_static, d_chunks_weighted, d_stage,
                     d_Tv, d_Kbar, d_ckpt, d_Unod, d_L, d_Vt, d_fnrm, d_DW, d_Vtb, d_sstore, d_ckpt_q,
@@ -1161,6 +1171,12 @@ dg_status dg_batch_layout(const dg_mesh* mesh, int64_t* instance_elem_off, int64
 
 namespace {
 
+// Warps per element for n points per direction: the lines of a pass (5 n^2
+// lanes' worth of work) per block.  Measured on mixed meshes (step, two warps
+// / chosen): n = 4 1848 / 1805 us, n = 5 7058 / 6406 us, n = 6 viscous
+// 4394 / 3508 us; n <= 3 is within 2% from two to four warps.
+int default_warps(int n) { return n <= 3 ? 2 : (n == 4 ? 3 : 4); }
+
 dg_status create_device_mesh(dg_mesh* m, const dg_mesh_desc* desc, cudaStream_t stream, dg_mesh** out) {
   m->flux = desc->flux;
   m->gamma = desc->gamma;
@@ -1170,7 +1186,7 @@ dg_status create_device_mesh(dg_mesh* m, const dg_mesh_desc* desc, cudaStream_t 
   cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, m->device);
   const dgh::HostMesh& h = m->h;
   m->nQmax = h.n * h.n * h.n;
-  m->wpb = m->nQmax >= 216 ? 1 : 2;  // warps cooperating on one element
+  m->wpb = default_warps(h.n);  // warps cooperating on one element
   auto fail_cuda = [&](cudaError_t e, const char* what) {
     m->release();
     delete m;
@@ -1182,6 +1198,7 @@ dg_status create_device_mesh(dg_mesh* m, const dg_mesh_desc* desc, cudaStream_t 
   std::vector<int> slot_tab(h.slot_tab);
   if ((e = upload(&m->d_dpool, h.tables.dpool)) != cudaSuccess) return fail_cuda(e, "upload tables");
   if ((e = upload(&m->d_ipool, h.tables.ipool)) != cudaSuccess) return fail_cuda(e, "upload tables");
+  if ((e = upload(&m->d_fpool, h.tables.fpool)) != cudaSuccess) return fail_cuda(e, "upload tables");
   if ((e = upload(&m->d_tabs, h.tables.tabs)) != cudaSuccess) return fail_cuda(e, "upload tables");
   if ((e = upload(&m->d_slot_tab, slot_tab)) != cudaSuccess) return fail_cuda(e, "upload slots");
   if ((e = upload(&m->d_slot_type, h.slot_type)) != cudaSuccess) return fail_cuda(e, "upload slots");
@@ -1220,7 +1237,7 @@ dg_status create_device_mesh(dg_mesh* m, const dg_mesh_desc* desc, cudaStream_t 
     const std::vector<double> w0 = m->static_weights();
     for (int t = 0; t < dgk::kMaxTabs; ++t) {
       m->weight[t] = w0[t];
-      m->tab_wpb[t] = m->wpb;
+      m->tab_wpb[t] = t < (int)h.tables.tabs.size() ? default_warps(h.tables.tabs[t].n) : m->wpb;
     }
   }
   if ((e = m->build_groups()) != cudaSuccess) return fail_cuda(e, "chunk table");

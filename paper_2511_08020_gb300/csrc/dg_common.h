@@ -21,6 +21,11 @@ constexpr int kNumTypes = 4;
 constexpr int kMaxTabs = kNumTypes * kMaxN;   // (type, N) tables, N = 1..kMaxN
 enum { HEX = 0, PRISM = 1, PYR = 2, TET = 3 };
 
+// A table coefficient of the fixed-point contractions.
+struct FixPair {
+  int x, y;
+};
+
 // Face descriptor of a local face: the face points are the tensor grid of
 // two collapsed coordinates (alpha, beta) with the third fixed at an end.
 struct FaceDesc {
@@ -54,6 +59,11 @@ struct TypeTab {
   int p_cbase, p_blen, p_boff;              // [n]
   int mode_col;                             // [nM]
   FaceDesc faces[6];
+  // fixed-point copies of B, C and ext in the pair pool, at the same offsets:
+  // coefficient c as round(c 2^59) = x 2^31 + y, the rows of B and C scaled by
+  // 2^-s to at most 1 first: s per column (B) and per mode (C) in the int pool
+  int col_s, mode_s;
+  int face_of[6];                           // local face at the end (2 l + end) of collapsed coordinate l, or -1
 };
 
 // Per-element geometry (affine): Jg = J * dxi/dx (row k = xi_k, column d = x_d)

@@ -1,0 +1,847 @@
+// Fixed-point contractions of the element kernels.
+//
+// FP64 issues 2 DFMA per clock and SM on this part (measured 1.71), the
+// 32 x 32 + 64 bit integer multiply-add 64 (measured 61).  A dot product of n
+// doubles with table coefficients is therefore done on integers: the n values
+// share one exponent (their largest), become 61-bit integers D = dh 2^31 + dl,
+// the coefficients are 62-bit integers C = ch 2^31 + cl, and
+//   sum C D / 2^62 = sum dh ch + (sum dh cl + dl ch) / 2^31
+// takes three multiply-adds per term (the dl cl products lie below the last
+// bit kept).  The last bit is 2^-61 of the largest input times the row's
+// growth, against 2^-53 of every partial sum in FP64, and the result is
+// rounded once, to nearest, when it becomes a double again; so the
+// contraction is as accurate as the FP64 chain or better for every input
+// whose block is finite.  A block that holds an infinity or a NaN gives NaN
+// throughout, zeros give zeros, and results below the normal range give zero.
+//
+// A value keeps its scale as `eb`: |x| < 2^(eb - 1023), x = R 2^(eb - 1084).
+// Between the passes of one transform the integers stay in shared memory,
+// every line with its own exponent, taken from its results (the OR of their
+// magnitudes): the collapsed bases grow towards the degenerate edge where the
+// weighted data shrink, so one exponent per element would cost the bits that
+// the next pass needs there (measured: 5 to 10 times the FP64 passes' error at
+// N = 6, with an exponent per line two thirds of it).  Sums of several
+// directions (the derivative sum, the lift) share one exponent per variable.
+//
+// A lane owns one line of n points of one variable: it reads the n values
+// once and forms all n results, so the coefficients are the same for every
+// lane of a pass (constant memory operands), except in the ragged passes
+// (prism and tetrahedron b, pyramid and tetrahedron c), which read theirs
+// from the table pool.
+#pragma once
+#include "dg_kernels.cuh"
+
+namespace dgk {
+namespace {
+
+// Tables per n: coefficient c is stored as round(c 2^(62 - g)) =
+// x 2^31 + y with -2^30 <= y < 2^30; g bounds every row (and column) sum of
+// |c| by 2^g, and 2^31 sum |x| + 2^30 sum |y| < 2^63 per row.
+//   A(p, i) = sqrt((2p + 1)/2) P_p(x_i)   (Legendre basis at the Gauss points)
+//   D(r, i) = l'_r(x_i)                   (collocation derivative, transposed)
+//   E(end, m) = l_m(-1), l_m(+1)          (extrapolation, g = kFxGE)
+// S(r) = 2^30 + sum_i y(D(r, i)) / 2: the half that makes a row's shift by 31
+// round to nearest, and the mean of the dl cl products that are not formed (dl
+// is uniform on [0, 2^31)): without it every derivative sum would lean the same
+// way, and the transform behind it adds the leanings up.
+constexpr int kFxGE = 3;
+constexpr int kFxGR = 3;   // growth of the ragged passes (rows scaled to at most 1, at most 7 terms)
+template <int n>
+struct FxTab;
+
+__constant__ int2 kFxA2[4] = {
+    {759250125, -12858223}, {759250125, -12858223}, {-759250125, 12858223}, {759250125, -12858223}};
+__constant__ int2 kFxD2[4] = {
+    {-929887697, 666064268}, {-929887697, 666064268}, {929887697, -666064268}, {929887697, -666064268}};
+__constant__ int2 kFxE2[4] = {
+    {366689652, 370354845}, {-98254196, -370354845}, {-98254196, -370354845}, {366689652, 370354845}};
+__constant__ long long kFxS2[2] = {1739806092, 407677556};
+template <> struct FxTab<2> {
+  static constexpr int gA = 1, gD = 1;
+  static __device__ __forceinline__ int2 A(int p, int i) { return kFxA2[p * 2 + i]; }
+  static __device__ __forceinline__ int2 D(int r, int i) { return kFxD2[r * 2 + i]; }
+  static __device__ __forceinline__ long long S(int r) { return kFxS2[r]; }
+  static __device__ __forceinline__ int2 E(int end, int m) { return kFxE2[end * 2 + m]; }
+};
+
+__constant__ int2 kFxA3[9] = {
+    {379625062, 1067312712}, {379625062, 1067312712}, {379625062, 1067312712}, {-509320467, -909560612}, {0, 0},
+    {509320467, 909560612}, {339546978, 606373742}, {-424433723, 315774647}, {339546978, 606373742}};
+__constant__ int2 kFxD3[9] = {
+    {-519823025, -665283801}, {-173274342, 494066616}, {173274342, -494066616}, {693097367, 171217185}, {0, 0},
+    {-693097367, -171217185}, {-173274342, 494066616}, {173274342, -494066616}, {519823025, 665283801}};
+__constant__ int2 kFxE3[6] = {
+    {396970555, 221761267}, {-178956971, 715827883}, {50421872, -937589150}, {50421872, -937589150},
+    {-178956971, 715827883}, {396970555, 221761267}};
+__constant__ long long kFxS3[3] = {741099923, 1073741824, 1406383724};
+template <> struct FxTab<3> {
+  static constexpr int gA = 2, gD = 3;
+  static __device__ __forceinline__ int2 A(int p, int i) { return kFxA3[p * 3 + i]; }
+  static __device__ __forceinline__ int2 D(int r, int i) { return kFxD3[r * 3 + i]; }
+  static __device__ __forceinline__ long long S(int r) { return kFxS3[r]; }
+  static __device__ __forceinline__ int2 E(int end, int m) { return kFxE3[end * 3 + m]; }
+};
+
+__constant__ int2 kFxA4[16] = {
+    {379625062, 1067312712}, {379625062, 1067312712}, {379625062, 1067312712}, {379625062, 1067312712},
+    {-566222869, -1000043699}, {-223547700, -546687481}, {223547700, 546687481}, {566222869, 1000043699},
+    {519790077, -989244199}, {-277256521, 808801544}, {-277256521, 808801544}, {519790077, -989244199},
+    {-306085893, 192663021}, {413536929, 955962303}, {-413536929, -955962303}, {306085893, -192663021}};
+__constant__ int2 kFxD4[16] = {
+    {-447213501, -899078943}, {-101677662, 241694245}, {44117129, -305844501}, {-77930594, 692007722},
+    {652318883, 864221711}, {-51595226, -718762622}, {-197390017, -171223876}, {283035976, -726864953},
+    {-283035976, 726864953}, {197390017, 171223876}, {51595226, 718762622}, {-652318883, -864221711},
+    {77930594, -692007722}, {-44117129, 305844501}, {101677662, -241694245}, {447213501, 899078943}};
+__constant__ int2 kFxE4[8] = {
+    {409844067, -703286682}, {-218407798, 870975805}, {107578601, 970901277}, {-30579415, 1008893247},
+    {-30579415, 1008893247}, {107578601, 970901277}, {-218407798, 870975805}, {409844067, -703286682}};
+__constant__ long long kFxS4[4] = {938131085, 697426954, 1450056694, 1209352562};
+template <> struct FxTab<4> {
+  static constexpr int gA = 2, gD = 4;
+  static __device__ __forceinline__ int2 A(int p, int i) { return kFxA4[p * 4 + i]; }
+  static __device__ __forceinline__ int2 D(int r, int i) { return kFxD4[r * 4 + i]; }
+  static __device__ __forceinline__ long long S(int r) { return kFxS4[r]; }
+  static __device__ __forceinline__ int2 E(int end, int m) { return kFxE4[end * 4 + m]; }
+};
+
+__constant__ int2 kFxA5[25] = {
+    {189812531, 533656356}, {189812531, 533656356}, {189812531, 533656356}, {189812531, 533656356},
+    {189812531, 533656356}, {-297920170, 83774255}, {-177029835, 524643203}, {0, 0}, {177029835, -524643203},
+    {297920170, -83774255}, {310576350, 839747701}, {-27620535, -334436249}, {-212216861, -915854501},
+    {-27620535, -334436249}, {310576350, 839747701}, {-251616227, -975912404}, {209607937, 905822449}, {0, 0},
+    {-209607937, -905822449}, {251616227, 975912404}, {139931009, -1020151954}, {-196171759, 1021104415},
+    {213539098, -741813879}, {-196171759, 1021104415}, {139931009, -1020151954}};
+__constant__ int2 kFxD5[25] = {
+    {-340043338, -464414026}, {-64441691, 225275681}, {20211053, 155274482}, {-16402521, -846373609},
+    {37028447, -942733549}, {516869255, 39386024}, {-50892223, 182790769}, {-96327274, -734527880},
+    {62314474, 700400628}, {-131560158, 751241848}, {-271357628, 233536301}, {161245867, -554039431}, {0, 0},
+    {-161245867, 554039431}, {271357628, -233536301}, {131560158, -751241848}, {-62314474, -700400628},
+    {96327274, 734527880}, {50892223, -182790769}, {-516869255, -39386024}, {-37028447, 942733549},
+    {16402521, 846373609}, {-20211053, -155274482}, {64441691, -225275681}, {340043338, 464414026}};
+__constant__ int2 kFxE5[10] = {
+    {416452927, 216256544}, {-239755380, -508451132}, {143165577, -1002159036}, {-71925040, 867629694},
+    {20497372, 426723931}, {20497372, 426723931}, {-71925040, 867629694}, {143165577, -1002159036},
+    {-239755380, -508451132}, {416452927, 216256544}};
+__constant__ long long kFxS5[5] = {137256313, 1543387518, 1073741824, 604096129, 2010227334};
+template <> struct FxTab<5> {
+  static constexpr int gA = 3, gD = 5;
+  static __device__ __forceinline__ int2 A(int p, int i) { return kFxA5[p * 5 + i]; }
+  static __device__ __forceinline__ int2 D(int r, int i) { return kFxD5[r * 5 + i]; }
+  static __device__ __forceinline__ long long S(int r) { return kFxS5[r]; }
+  static __device__ __forceinline__ int2 E(int end, int m) { return kFxE5[end * 5 + m]; }
+};
+
+__constant__ int2 kFxA6[36] = {
+    {189812531, 533656356}, {189812531, 533656356}, {189812531, 533656356}, {189812531, 533656356},
+    {189812531, 533656356}, {189812531, 533656356}, {-306563291, -819992555}, {-217382470, 897060234},
+    {-78449624, -672064299}, {78449624, 672064299}, {217382470, -897060234}, {306563291, 819992555},
+    {341350436, 813569934}, {66125407, -57509816}, {-175966540, 47828096}, {-175966540, 47828096},
+    {66125407, -57509816}, {341350436, 813569934}, {-315505072, -1040216138}, {135149066, -308332591},
+    {162692597, 18236024}, {-162692597, -18236024}, {-135149066, 308332591}, {315505072, 1040216138},
+    {240305517, 59302192}, {-243859293, -524105452}, {100028740, 957889305}, {100028740, 957889305},
+    {-243859293, -524105452}, {240305517, 59302192}, {-129503500, -417942196}, {185332979, 1038570682},
+    {-210655037, 834718133}, {210655037, -834718133}, {-185332979, -1038570682}, {129503500, 417942196}};
+__constant__ int2 kFxD6[36] = {
+    {-479514787, 597921728}, {-82095983, 547488998}, {21770942, 296410655}, {-12898916, -1049652637},
+    {13973559, 836191447}, {-35984482, 1034952997}, {745531409, -820203965}, {-78843002, 111654258},
+    {-107719820, -12926339}, {50588903, -123531274}, {-50747059, -823783667}, {126896921, -571362468},
+    {-429685754, 323554590}, {234112882, 664201462}, {-16980306, -271292391}, {-140619170, -962107812},
+    {109947398, -836546710}, {-254581571, -362318177}, {254581571, 362318177}, {-109947398, 836546710},
+    {140619170, 962107812}, {16980306, 271292391}, {-234112882, -664201462}, {429685754, -323554590},
+    {-126896921, 571362468}, {50747059, 823783667}, {-50588903, 123531274}, {107719820, 12926339},
+    {78843002, -111654258}, {-745531409, 820203965}, {35984482, -1034952997}, {-13973559, -836191447},
+    {12898916, 1049652637}, {-21770942, -296410655}, {82095983, -547488998}, {479514787, -597921728}};
+__constant__ int2 kFxE6[12] = {
+    {420282199, 922413512}, {-252453572, -341664032}, {165605901, -537754574}, {-101798161, -311317499},
+    {51485924, 492366964}, {-14686835, -224044369}, {-14686835, -224044369}, {51485924, 492366964},
+    {-101798161, -311317499}, {165605901, -537754574}, {-252453572, -341664032}, {420282199, 922413512}};
+__constant__ long long kFxS6[6] = {2205398418, -46334904, 351487305, 1795996343, 2193818551, -57914770};
+template <> struct FxTab<6> {
+  static constexpr int gA = 3, gD = 5;
+  static __device__ __forceinline__ int2 A(int p, int i) { return kFxA6[p * 6 + i]; }
+  static __device__ __forceinline__ int2 D(int r, int i) { return kFxD6[r * 6 + i]; }
+  static __device__ __forceinline__ long long S(int r) { return kFxS6[r]; }
+  static __device__ __forceinline__ int2 E(int end, int m) { return kFxE6[end * 6 + m]; }
+};
+
+__constant__ int2 kFxA7[49] = {
+    {189812531, 533656356}, {189812531, 533656356}, {189812531, 533656356}, {189812531, 533656356},
+    {189812531, 533656356}, {189812531, 533656356}, {189812531, 533656356}, {-312033413, -1034234961},
+    {-243789462, 643368571}, {-133427660, -221439034}, {0, 0}, {133427660, 221439034}, {243789462, -643368571},
+    {312033413, 1034234961}, {361281696, 218237818}, {137857240, -265157790}, {-107353961, -79373268},
+    {-212216861, -915854501}, {-107353961, -79373268}, {137857240, -265157790}, {361281696, 218237818},
+    {-358439408, -273523909}, {46671745, -678880659}, {221795472, -575145396}, {0, 0}, {-221795472, 575145396},
+    {-46671745, 678880659}, {358439408, 273523909}, {311526146, -95167372}, {-207390392, -1020774108},
+    {-70594378, -580867171}, {213539098, -741813879}, {-70594378, -580867171}, {-207390392, -1020774108},
+    {311526146, -95167372}, {-228917650, 221160001}, {259226256, 462864617}, {-165414722, 379312394}, {0, 0},
+    {165414722, -379312394}, {-259226256, -462864617}, {228917650, -221160001}, {121017149, -541844870},
+    {-175401296, -1007889148}, {204501750, -43865357}, {-213868379, -900660478}, {204501750, -43865357},
+    {-175401296, -1007889148}, {121017149, -541844870}};
+__constant__ int2 kFxD7[49] = {
+    {-321054924, 845902738}, {-51630206, -423505199}, {12394788, -1070654788}, {-6197551, -47878989},
+    {4969638, 389777488}, {-6339158, -1067834623}, {17676827, -839016535}, {506102643, -669638213},
+    {-55276420, 713080389}, {-62803395, -39058071}, {24835543, -306580161}, {-18374287, -929670968},
+    {22625098, 740676974}, {-62139300, 169420688}, {-307780304, -679006439}, {159092650, -688963064},
+    {-16303210, 177762420}, {-72223114, -1022541253}, {41338959, -387006813}, {-46545479, 1035353814},
+    {123403225, 169384752}, {201673337, 2530819}, {-82445562, -1039899609}, {94646127, 5050145}, {0, 0},
+    {-94646127, -5050145}, {82445562, 1039899609}, {-201673337, -2530819}, {-123403225, -169384752},
+    {46545479, -1035353814}, {-41338959, 387006813}, {72223114, 1022541253}, {16303210, -177762420},
+    {-159092650, 688963064}, {307780304, 679006439}, {62139300, -169420688}, {-22625098, -740676974},
+    {18374287, 929670968}, {-24835543, 306580161}, {62803395, 39058071}, {55276420, -713080389},
+    {-506102643, 669638213}, {-17676827, 839016535}, {6339158, 1067834623}, {-4969638, -389777488},
+    {6197551, 47878989}, {-12394788, 1070654788}, {51630206, 423505199}, {321054924, -845902738}};
+__constant__ int2 kFxE7[14] = {
+    {422695246, 334795903}, {-260577463, -919111227}, {180417580, 851078313}, {-122713351, -674923432},
+    {76250204, 892527342}, {-38673524, 87890175}, {11036764, -572257074}, {11036764, -572257074},
+    {-38673524, 87890175}, {76250204, 892527342}, {-122713351, -674923432}, {180417580, 851078313},
+    {-260577463, -919111227}, {422695246, 334795903}};
+__constant__ long long kFxS7[7] = {-32863130, 912857143, 376233532, 1073741824, 1771250115, 1234626505, 2180346778};
+template <> struct FxTab<7> {
+  static constexpr int gA = 3, gD = 6;
+  static __device__ __forceinline__ int2 A(int p, int i) { return kFxA7[p * 7 + i]; }
+  static __device__ __forceinline__ int2 D(int r, int i) { return kFxD7[r * 7 + i]; }
+  static __device__ __forceinline__ long long S(int r) { return kFxS7[r]; }
+  static __device__ __forceinline__ int2 E(int end, int m) { return kFxE7[end * 7 + m]; }
+};
+
+// Exponent bookkeeping in shared memory: sets of five words (one per variable).
+__device__ __forceinline__ unsigned* fx_slots() {
+  __shared__ unsigned s[15];
+  return s;
+}
+
+struct FxD {
+  int h, l;   // D = h 2^31 + l, 0 <= l < 2^31
+};
+
+// D 2^k as (h, l), 0 <= k <= 29
+__device__ __forceinline__ FxD fx_split(long long D, int k) {
+  const unsigned lo = (unsigned)D, hi = (unsigned)((unsigned long long)D >> 32);
+  FxD f;
+  f.h = (int)__funnelshift_r(lo, hi, 31 - k);
+  f.l = (int)((lo << k) & 0x7fffffffu);
+  return f;
+}
+
+// x 2^(1083 - em) as an integer, |x| < 2^(em + 1 - 1023); neg: of -x.  A
+// subnormal x counts half (its exponent field is that of no hidden bit).
+__device__ __forceinline__ long long fx_from(double x, int em, unsigned neg = 0u) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), e = (hi >> 20) & 0x7ffu;
+  const int d = min(em - (int)e, 63);
+  const unsigned mh = (__funnelshift_l(lo, hi, 8) & 0x0fffffffu) | (min(e, 1u) << 28), ml = lo << 8;
+  const unsigned long long M = (((unsigned long long)mh << 32) | ml) >> d;
+  const long long s = (long long)((int)(hi ^ neg) >> 31);
+  return ((long long)M ^ s) - s;
+}
+
+constexpr int kFxBad = 1 << 19;   // added to the exponent of a block with an infinity or a NaN
+
+// R 2^(eb - 1084) rounded to nearest (zero below the normal range, infinity
+// above it, NaN for a block that held an infinity or a NaN)
+__device__ __forceinline__ double fx_to(long long R, int eb) {
+  const int s = (int)(R >> 32) >> 31;
+  const unsigned long long a = (unsigned long long)((R ^ (long long)s) - (long long)s);
+  const unsigned a1 = (unsigned)(a >> 32), a0 = (unsigned)a;
+  const bool low = a1 == 0u;
+  const unsigned ah = low ? a0 : a1, al = low ? 0u : a0;
+  const int z = __clz((int)ah);
+  const int e = (low ? eb - 31 : eb + 1) - z;
+  const unsigned nh = __funnelshift_l(al, ah, z), nl = __funnelshift_l(0u, al, z);
+  const unsigned long long t =
+      (((unsigned long long)((nh >> 11) + ((unsigned)e << 20)) << 32) | __funnelshift_r(nl, nh, 11)) +
+      (unsigned long long)((nl >> 10) & 1u);
+  unsigned th = (unsigned)(t >> 32), tl = (unsigned)t;
+  if (nh == 0u || (unsigned)e >= 2046u) {
+    tl = 0u;
+    th = eb >= kFxBad ? 0x7ff80000u : (e >= 2046 ? 0x7ff00000u : 0u);
+  }
+  return __hiloint2double((int)(th | ((unsigned)s & 0x80000000u)), (int)tl);
+}
+
+// exponent of a block from the largest high word (sign cleared) of its values
+__device__ __forceinline__ int fx_em(unsigned hmax) {
+  const int e = (int)(hmax >> 20);
+  return e == 2047 ? kFxBad + 2047 : e;
+}
+
+// shift that brings integers with OR of high words (one's complement) m to 61 bits
+__device__ __forceinline__ int fx_shift(unsigned m) { return max(__clz((int)m) - 3, 0); }
+
+__device__ __forceinline__ unsigned fx_mag(long long R) {
+  const int h = (int)(R >> 32);
+  return (unsigned)(h ^ (h >> 31));
+}
+
+// a b + c, one instruction (written out: the C++ expression on operands that
+// the compiler has already widened becomes a three-instruction 64-bit product)
+__device__ __forceinline__ long long fx_madw(int a, int b, long long c) {
+  long long r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
+
+__device__ __forceinline__ unsigned fx_hi(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+
+// Block maximum of every lane's five m[v] into slot[v] (zero before; a
+// barrier must follow).
+__device__ __forceinline__ void fx_flush_max(const unsigned* m, unsigned* slot) {
+  const int l32 = threadIdx.x & 31;
+  unsigned x = 0u;
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    const unsigned r = __reduce_max_sync(0xffffffffu, m[v]);
+    x = l32 == v ? r : x;
+  }
+  if (l32 < 5) atomicMax(slot + l32, x);
+}
+
+// Largest high words of buf[v stride + i], i < cnt, into m[v]
+__device__ __forceinline__ void fx_scan(const double* buf, int cnt, int stride, unsigned* m) {
+#pragma unroll
+  for (int v = 0; v < 5; ++v)
+    for (int q = threadIdx.x; q < cnt; q += blockDim.x) m[v] = max(m[v], fx_hi(buf[v * stride + q]));
+}
+
+__device__ __forceinline__ void fx_clear(unsigned* slot, int cnt) {
+  for (int t = threadIdx.x; t < cnt; t += blockDim.x) slot[t] = 0u;
+}
+
+// Exponents of the lines between two passes
+template <int n>
+__device__ __forceinline__ int* fx_exps() {
+  __shared__ int e[10 * n * n];
+  return e;
+}
+
+// One lane's results R[0..n) of scale eb, brought to 61 bits and stored with
+// the given stride; returns their exponent.
+template <int n>
+__device__ __forceinline__ int fx_store_line(const long long* R, int eb, long long* o, int stride) {
+  unsigned mg = 0u;
+#pragma unroll
+  for (int i = 0; i < n; ++i) mg |= fx_mag(R[i]);
+  const int k = fx_shift(mg);
+#pragma unroll
+  for (int i = 0; i < n; ++i) o[i * stride] = R[i] << k;
+  return eb - k;
+}
+
+// The integers x[i stride] of exponents e[i estride] on the largest of them;
+// returns it.
+template <int n>
+__device__ __forceinline__ int fx_load_aligned(const long long* x, int stride, const int* e, int estride, FxD* d) {
+  int ei[n], em = e[0];
+#pragma unroll
+  for (int i = 0; i < n; ++i) {
+    ei[i] = e[i * estride];
+    em = max(em, ei[i]);
+  }
+#pragma unroll
+  for (int i = 0; i < n; ++i) d[i] = fx_split(x[i * stride] >> min(em - ei[i], 63), 0);
+  return em;
+}
+
+constexpr long long kFxHalf = 1ll << 30;   // rounds a sum's shift by 31 to nearest
+
+// sum_m C(m) D_m 2^-62 over n terms; C(m) yields the coefficient pair
+template <int n, class Coef>
+__device__ __forceinline__ long long fx_dot(const FxD* d, Coef C, long long mid = kFxHalf) {
+#pragma unroll
+  for (int m = 0; m < n; ++m) {
+    const int2 k = C(m);
+    mid = fx_madw(d[m].h, k.y, mid);
+    mid = fx_madw(d[m].l, k.x, mid);
+  }
+  long long hh = mid >> 31;
+#pragma unroll
+  for (int m = 0; m < n; ++m) hh = fx_madw(d[m].h, C(m).x, hh);
+  return hh;
+}
+
+// Exponent of n doubles (their largest) and their integers
+template <int n>
+__device__ __forceinline__ int fx_line(const double* x, FxD* d) {
+  unsigned m = 0u;
+#pragma unroll
+  for (int i = 0; i < n; ++i) m = max(m, (unsigned)__double2hiint(x[i]) & 0x7fffffffu);
+  const int em = fx_em(m);
+#pragma unroll
+  for (int i = 0; i < n; ++i) d[i] = fx_split(fx_from(x[i], em), 0);
+  return em;
+}
+
+// ragged pass: outputs o < n of sum_t tab[t n + o] D_t, t < len
+template <int n, class Load>
+__device__ __forceinline__ void fx_ragged_out(const int2* tab, int len, Load load, long long* R) {
+  long long mid[n], hh[n];
+#pragma unroll
+  for (int o = 0; o < n; ++o) {
+    mid[o] = kFxHalf;
+    hh[o] = 0;
+  }
+#pragma unroll 1
+  for (int t = 0; t < len; ++t) {
+    const FxD d = load(t);
+#pragma unroll
+    for (int o = 0; o < n; ++o) {
+      const int2 k = __ldg(tab + t * n + o);
+      mid[o] = fx_madw(d.h, k.y, mid[o]);
+      mid[o] = fx_madw(d.l, k.x, mid[o]);
+      hh[o] = fx_madw(d.h, k.x, hh[o]);
+    }
+  }
+#pragma unroll
+  for (int o = 0; o < n; ++o) R[o] = hh[o] + (mid[o] >> 31);
+}
+
+// Line `id` of direction l: start index and stride in the nodal block, and
+// the two other indices (x1 < x2 by coordinate; face point x1 + n x2)
+template <int n>
+__device__ __forceinline__ void fx_line_of(int l, int id, int& start, int& stride, int& fp) {
+  const int x1 = id / n, x2 = id - x1 * n;
+  start = l == 0 ? id : (l == 1 ? x1 * n * n + x2 : id * n);
+  stride = l == 0 ? n * n : (l == 1 ? n : 1);
+  fp = x1 + n * x2;
+}
+
+// The face values at both ends of one line of direction l
+template <int n, class Out>
+__device__ __forceinline__ void fx_line_ends(const TypeTab& T, int l, int v, int fp, const double* x, Out out) {
+  using Tab = FxTab<n>;
+  FxD d[n];
+  const int eb = fx_line<n>(x, d) + 1 + kFxGE;
+  const int lf0 = __ldg(&T.face_of[2 * l]), lf1 = __ldg(&T.face_of[2 * l + 1]);
+  if (lf0 >= 0) out(lf0, v, fp, fx_to(fx_dot<n>(d, [&](int m) { return Tab::E(0, m); }), eb));
+  if (lf1 >= 0) out(lf1, v, fp, fx_to(fx_dot<n>(d, [&](int m) { return Tab::E(1, m); }), eb));
+}
+
+// Values of the nodal field src [5][nQ] on the element's own face points:
+// out(local face, variable, face point, value), directions l0..2.  The faces
+// at both ends of a coordinate share the line's integers.
+template <int n, class Out>
+__device__ __forceinline__ void fx_traces(const TypeTab& T, const double* src, Out out, int l0 = 0) {
+  constexpr int n2 = n * n, nQ = n2 * n;
+#pragma unroll 1
+  for (int t0 = l0 * 5 * n2 + threadIdx.x; t0 < 15 * n2; t0 += blockDim.x) {
+    const int l = t0 / (5 * n2), r = t0 - l * 5 * n2, v = r / n2;
+    int st, sd, fp;
+    fx_line_of<n>(l, r - v * n2, st, sd, fp);
+    const double* s = src + v * nQ + st;
+    double x[n];
+#pragma unroll
+    for (int m = 0; m < n; ++m) x[m] = s[m * sd];
+    fx_line_ends<n>(T, l, v, fp, x, out);
+  }
+}
+
+// Modal -> nodal, U = V Q: sQ [5][nM] doubles -> bufA [5][nQ] doubles, bufB
+// [5][nQ] scratch (sQ may alias bufB).  Passes c, b, a, one line per lane.
+// TR: the values at the element's face points too, out(local face, variable,
+// face point, value), bit for bit fx_traces of U (the a faces by the lane that
+// forms the line).
+template <int n, bool TR, class Out>
+__device__ __forceinline__ void fx_to_nodal(const Ctx& c, const TypeTab& T, const double* sQ, double* bufA,
+                                            double* bufB, Out out) {
+  constexpr int n2 = n * n, nQ = n2 * n;
+  using Tab = FxTab<n>;
+  int* e0 = fx_exps<n>();
+  int* e1 = e0 + 5 * n2;
+  const int* ip = c.ipool;
+  const int nM = T.nM, ncols = T.ncols, nt = blockDim.x;
+  long long* X = reinterpret_cast<long long*>(bufA);
+  long long* Y = reinterpret_cast<long long*>(bufB);
+  const bool uc = T.type == HEX || T.type == PRISM, ub = T.type == HEX || T.type == PYR;
+  // c-pass: X[col][k] = sum_t C[col][t][k] Q[moff[col] + t]
+  for (int t0 = threadIdx.x; t0 < 5 * ncols; t0 += nt) {
+    const int v = t0 / ncols, col = t0 - v * ncols;
+    long long R[n];
+    int eb;
+    if (uc) {
+      const double* q = sQ + v * nM + col * n;
+      double x[n];
+#pragma unroll
+      for (int t = 0; t < n; ++t) x[t] = q[t];
+      FxD d[n];
+      eb = fx_line<n>(x, d) + 1 + Tab::gA;
+#pragma unroll
+      for (int k = 0; k < n; ++k) R[k] = fx_dot<n>(d, [&](int t) { return Tab::A(t, k); });
+    } else {
+      const double* q = sQ + v * nM + __ldg(ip + T.col_moff + col);
+      const int len = __ldg(ip + T.col_len + col);
+      const int* ms = ip + T.mode_s + (q - sQ - v * nM);
+      int em = fx_em(fx_hi(q[0])) + __ldg(ms);
+      for (int t = 1; t < len; ++t) em = max(em, fx_em(fx_hi(q[t])) + __ldg(ms + t));
+      eb = em + 1 + kFxGR;
+      fx_ragged_out<n>(c.fpool + T.C + __ldg(ip + T.col_coff + col), len,
+                       [&](int t) { return fx_split(fx_from(q[t], em - __ldg(ms + t)), 0); }, R);
+    }
+    e0[v * n2 + col] = fx_store_line<n>(R, eb, X + v * nQ + col * n, 1);
+  }
+  __syncthreads();
+  // b-pass: Y[p][j][k] = sum_t B[p][t][j] X[cbase[p] + t][k]
+  for (int t0 = threadIdx.x; t0 < 5 * n2; t0 += nt) {
+    const int v = t0 / n2, pk = t0 - v * n2, p = pk / n, k = pk - p * n;
+    const int cb = __ldg(ip + T.p_cbase + p);
+    long long R[n];
+    int eb;
+    const long long* x = X + v * nQ + cb * n + k;
+    const int* e = e0 + v * n2 + cb;
+    if (ub) {
+      FxD d[n];
+      eb = fx_load_aligned<n>(x, n, e, 1, d) + Tab::gA;
+#pragma unroll
+      for (int j = 0; j < n; ++j) R[j] = fx_dot<n>(d, [&](int t) { return Tab::A(t, j); });
+    } else {
+      const int len = __ldg(ip + T.p_blen + p);
+      const int* cs = ip + T.col_s + cb;
+      int em = e[0] + __ldg(cs);
+      for (int t = 1; t < len; ++t) em = max(em, e[t] + __ldg(cs + t));
+      eb = em + kFxGR;
+      fx_ragged_out<n>(c.fpool + T.B + __ldg(ip + T.p_boff + p), len,
+                       [&](int t) { return fx_split(x[t * n] >> min(em - e[t] - __ldg(cs + t), 63), 0); }, R);
+    }
+    e1[v * n2 + pk] = fx_store_line<n>(R, eb, Y + v * nQ + p * n2 + k, n);
+  }
+  __syncthreads();
+  // a-pass: U[i][j][k] = sum_p A[p][i] Y[p][j][k]
+  for (int t0 = threadIdx.x; t0 < 5 * n2; t0 += nt) {
+    const int v = t0 / n2, jk = t0 - v * n2, j = jk / n, k = jk - j * n;
+    FxD d[n];
+    const int eb = fx_load_aligned<n>(Y + v * nQ + jk, n2, e1 + v * n2 + k, n, d) + Tab::gA;
+    double* o = bufA + v * nQ + jk;
+#pragma unroll
+    for (int i = 0; i < n; ++i) o[i * n2] = fx_to(fx_dot<n>(d, [&](int p) { return Tab::A(p, i); }), eb);
+    if (TR) {
+      double x[n];
+#pragma unroll
+      for (int i = 0; i < n; ++i) x[i] = o[i * n2];
+      fx_line_ends<n>(T, 0, v, j + n * k, x, out);
+    }
+  }
+  __syncthreads();
+  if (TR) {
+    fx_traces<n>(T, bufA, out, 1);
+    __syncthreads();
+  }
+}
+
+// The b and c passes of V^T: Y [5][nQ] (integers of the a-pass, their lines'
+// exponents in fx_exps) -> r [5][nM] doubles.  X [5][nQ] scratch; r may alias Y.
+template <int n>
+__device__ __forceinline__ void fx_modal_tail(const Ctx& c, const TypeTab& T, const long long* Y, long long* X,
+                                              double* r) {
+  constexpr int n2 = n * n, nQ = n2 * n;
+  using Tab = FxTab<n>;
+  const int* e0 = fx_exps<n>();
+  int* e1 = fx_exps<n>() + 5 * n2;
+  const int* ip = c.ipool;
+  const int nM = T.nM, ncols = T.ncols, nt = blockDim.x;
+  const bool uc = T.type == HEX || T.type == PRISM, ub = T.type == HEX || T.type == PYR;
+  // b-pass: X[cbase[p] + t][k] = sum_j B[p][t][j] Y[p][j][k]
+  for (int t0 = threadIdx.x; t0 < 5 * n2; t0 += nt) {
+    const int v = t0 / n2, pk = t0 - v * n2, p = pk / n, k = pk - p * n;
+    FxD d[n];
+    int eb = fx_load_aligned<n>(Y + v * nQ + p * n2 + k, n, e0 + v * n2 + k, n, d);
+    long long* o = X + v * nQ + __ldg(ip + T.p_cbase + p) * n + k;
+    if (ub) {
+      long long R[n];
+#pragma unroll
+      for (int t = 0; t < n; ++t) R[t] = fx_dot<n>(d, [&](int j) { return Tab::A(t, j); });
+      eb = fx_store_line<n>(R, eb + Tab::gA, o, n);
+    } else {
+      const int2* B = c.fpool + T.B + __ldg(ip + T.p_boff + p);
+      const int len = __ldg(ip + T.p_blen + p);
+      unsigned mg = 0u;
+#pragma unroll 1
+      for (int t = 0; t < len; ++t) {
+        const long long R = fx_dot<n>(d, [&](int j) { return __ldg(B + t * n + j); });
+        o[t * n] = R;
+        mg |= fx_mag(R);
+      }
+      const int s = fx_shift(mg);
+      for (int t = 0; t < len; ++t) o[t * n] <<= s;
+      eb += kFxGR - s;
+    }
+    e1[v * n2 + pk] = eb;
+  }
+  __syncthreads();
+  // c-pass: r[moff[col] + t] = sum_k C[col][t][k] X[col][k]
+  for (int t0 = threadIdx.x; t0 < 5 * ncols; t0 += nt) {
+    const int v = t0 / ncols, col = t0 - v * ncols;
+    FxD d[n];
+    // ub: the b-pass used the unscaled table
+    const int em = fx_load_aligned<n>(X + v * nQ + col * n, 1, e1 + v * n2 + __ldg(ip + T.col_p + col) * n, 1, d) +
+                   (ub ? 0 : __ldg(ip + T.col_s + col));
+    if (uc) {
+      double* o = r + v * nM + col * n;
+#pragma unroll
+      for (int t = 0; t < n; ++t) o[t] = fx_to(fx_dot<n>(d, [&](int k) { return Tab::A(t, k); }), em + Tab::gA);
+    } else {
+      const int2* C = c.fpool + T.C + __ldg(ip + T.col_coff + col);
+      const int len = __ldg(ip + T.col_len + col), mo = __ldg(ip + T.col_moff + col);
+      const int* ms = ip + T.mode_s + mo;
+      double* o = r + v * nM + mo;
+#pragma unroll 1
+      for (int t = 0; t < len; ++t)
+        o[t] = fx_to(fx_dot<n>(d, [&](int k) { return __ldg(C + t * n + k); }), em + kFxGR + __ldg(ms + t));
+    }
+  }
+  __syncthreads();
+}
+
+// Nodal -> modal transpose, r = V^T h: bufA [5][nQ] doubles (destroyed) ->
+// r [5][nM] doubles; bufB [5][nQ] scratch (r may alias bufB, not bufA).
+template <int n>
+__device__ __forceinline__ void fx_to_modal(const TypeTab& T, const Ctx& c, double* bufA, double* bufB, double* r) {
+  constexpr int n2 = n * n, nQ = n2 * n;
+  using Tab = FxTab<n>;
+  int* e0 = fx_exps<n>();
+  long long* Y = reinterpret_cast<long long*>(bufB);
+  // a-pass: Y[p][j][k] = sum_i A[p][i] h[i][j][k]
+  for (int t0 = threadIdx.x; t0 < 5 * n2; t0 += blockDim.x) {
+    const int v = t0 / n2, jk = t0 - v * n2;
+    const double* h = bufA + v * nQ + jk;
+    double x[n];
+#pragma unroll
+    for (int i = 0; i < n; ++i) x[i] = h[i * n2];
+    FxD d[n];
+    const int eb = fx_line<n>(x, d) + 1 + Tab::gA;
+    long long R[n];
+#pragma unroll
+    for (int p = 0; p < n; ++p) R[p] = fx_dot<n>(d, [&](int i) { return Tab::A(p, i); });
+    e0[v * n2 + jk] = fx_store_line<n>(R, eb, Y + v * nQ + jk, n2);
+  }
+  __syncthreads();
+  fx_modal_tail<n>(c, T, Y, reinterpret_cast<long long*>(bufA), r);
+}
+
+// r = V^T (H +- sum_f E_f^T F_f) of a prism, pyramid or tetrahedron: H(o) the
+// nodal value at v nQ + q, F(f, v, p) the face values (read once each); neg
+// 0x80000000 subtracts.  The sum stays in integers between the lift and the
+// transform: a lane owns the line (j, k), takes its n values of H, adds the b
+// and c face values with the two end coefficients of its j and k and the a
+// face values with the line's, and goes on with the a-pass.  bufA, bufG
+// [5][nQ] and F's [nf][5][n^2] at bufG (scratch); r [5][nM] may be bufA or lie
+// behind bufG's first 5 nQ.
+template <int n, class LoadH, class LoadF>
+__device__ __forceinline__ void fx_lift_to_modal(const Ctx& c, const TypeTab& T, LoadH H, LoadF F, unsigned neg,
+                                                 double* bufA, double* bufG, double* r) {
+  constexpr int n2 = n * n, nQ = n2 * n;
+  using Tab = FxTab<n>;
+  unsigned* sx = fx_slots();
+  int* e0 = fx_exps<n>();
+  const int nf = T.nfaces, nt = blockDim.x;
+  long long* Y = reinterpret_cast<long long*>(bufA);
+  long long* FI = reinterpret_cast<long long*>(bufG);
+  fx_clear(sx, 5);
+  unsigned m[5] = {0u, 0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    for (int q = threadIdx.x; q < nQ; q += nt) m[v] = max(m[v], fx_hi(H(v * nQ + q)));
+    for (int w = threadIdx.x; w < nf * n2; w += nt) {
+      const int lf = w / n2, p = w - lf * n2;
+      const double x = F(lf, v, p);
+      bufG[(lf * 5 + v) * n2 + p] = x;
+      m[v] = max(m[v], fx_hi(x));
+    }
+  }
+  __syncthreads();
+  fx_flush_max(m, sx);
+  __syncthreads();
+  // the face values as integers, in place (each lane the values it stored)
+  for (int v = 0; v < 5; ++v) {
+    const int em = fx_em(sx[v]);
+    for (int w = threadIdx.x; w < nf * n2; w += nt) {
+      const int lf = w / n2, o = lf * 5 * n2 + v * n2 + w - lf * n2;
+      FI[o] = fx_from(bufG[o], em, neg);
+    }
+  }
+  __syncthreads();
+  const int fa0 = __ldg(&T.face_of[0]), fa1 = __ldg(&T.face_of[1]);
+  const int2* E = c.fpool + T.ext;
+  for (int t0 = threadIdx.x; t0 < 5 * n2; t0 += nt) {
+    const int v = t0 / n2, jk = t0 - v * n2, j = jk / n, k = jk - j * n;
+    const int em = fx_em(sx[v]);
+    long long mid[n], hh[n], half = kFxHalf;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      hh[i] = fx_from(H(v * nQ + jk + i * n2), em + kFxGE);
+      mid[i] = 0;
+    }
+    // b faces (line value at (i, k), coefficient of j), then c faces ((i, j), of k)
+#pragma unroll 1
+    for (int e = 0; e < 4; ++e) {
+      const int lf = __ldg(&T.face_of[2 + e]);
+      if (lf < 0) continue;
+      const int2 co = __ldg(E + (e & 1) * n + (e < 2 ? j : k));
+      const long long* f = FI + (lf * 5 + v) * n2 + n * (e < 2 ? k : j);
+      half += co.y >> 1;   // the mean of the dl cl products (S above)
+#pragma unroll
+      for (int i = 0; i < n; ++i) {
+        const FxD d = fx_split(f[i], 0);
+        mid[i] = fx_madw(d.h, co.y, mid[i]);
+        mid[i] = fx_madw(d.l, co.x, mid[i]);
+        hh[i] = fx_madw(d.h, co.x, hh[i]);
+      }
+    }
+    unsigned mg = 0u;
+    {
+      const FxD a0 = fx_split(FI[(fa0 * 5 + v) * n2 + j + n * k], 0), a1 = fx_split(FI[(fa1 * 5 + v) * n2 + j + n * k], 0);
+#pragma unroll
+      for (int i = 0; i < n; ++i) {
+        const int2 c0 = Tab::E(0, i), c1 = Tab::E(1, i);
+        mid[i] = fx_madw(a0.h, c0.y, mid[i]);
+        mid[i] = fx_madw(a0.l, c0.x, mid[i]);
+        mid[i] = fx_madw(a1.h, c1.y, mid[i]);
+        mid[i] = fx_madw(a1.l, c1.x, mid[i]);
+        hh[i] = fx_madw(a0.h, c0.x, hh[i]);
+        hh[i] = fx_madw(a1.h, c1.x, hh[i]);
+        hh[i] += (mid[i] + half + ((c0.y + c1.y) >> 1)) >> 31;
+        mg |= fx_mag(hh[i]);
+      }
+    }
+    const int ks = fx_shift(mg);
+    FxD d[n];
+#pragma unroll
+    for (int i = 0; i < n; ++i) d[i] = fx_split(hh[i], ks);
+    long long R[n];
+#pragma unroll
+    for (int p = 0; p < n; ++p) R[p] = fx_dot<n>(d, [&](int i) { return Tab::A(p, i); });
+    e0[v * n2 + jk] = fx_store_line<n>(R, em + 1 + kFxGE + Tab::gA - ks, Y + v * nQ + jk, n2);
+  }
+  __syncthreads();
+  fx_modal_tail<n>(c, T, Y, FI, r);
+}
+
+// out = sum over the directions l in `dirs` of D_l^T G_l (collocation
+// derivative, G_l at G + 5 l nQ): out [5][nQ] (shared or global).  tmp
+// [5][nQ] scratch.  slot: set whose words hold the largest high word per
+// variable when `scanned`, else cleared and filled here.
+template <int n>
+__device__ __forceinline__ void fx_dsum_body(const double* G, unsigned dirs, double* tmp, double* out, unsigned* slot,
+                                             bool scanned) {
+  constexpr int n2 = n * n, nQ = n2 * n;
+  using Tab = FxTab<n>;
+  if (!scanned) {
+    fx_clear(slot, 5);
+    __syncthreads();
+    unsigned m[5] = {0u, 0u, 0u, 0u, 0u};
+#pragma unroll 1
+    for (int l = 0; l < 3; ++l)
+      if ((dirs >> l) & 1u) fx_scan(G + 5 * l * nQ, nQ, nQ, m);
+    fx_flush_max(m, slot);
+  }
+  __syncthreads();
+  long long* A = reinterpret_cast<long long*>(tmp);
+  bool first = true;
+#pragma unroll 1
+  for (int l = 2; l >= 0; --l) {
+    if (!((dirs >> l) & 1u)) continue;
+    const bool last = (dirs & ((1u << l) - 1u)) == 0u;
+    for (int t0 = threadIdx.x; t0 < 5 * n2; t0 += blockDim.x) {
+      const int v = t0 / n2;
+      int st, sd, fp;
+      fx_line_of<n>(l, t0 - v * n2, st, sd, fp);
+      const int em = fx_em(slot[v]) + 2;     // room for the three sums
+      const double* s = G + (5 * l + v) * nQ + st;
+      FxD d[n];
+#pragma unroll
+      for (int m = 0; m < n; ++m) d[m] = fx_split(fx_from(s[m * sd], em), 0);
+      const int o = v * nQ + st;
+#pragma unroll
+      for (int i = 0; i < n; ++i) {
+        long long R = fx_dot<n>(d, [&](int m) { return Tab::D(i, m); }, Tab::S(i));
+        if (!first) R += A[o + i * sd];
+        if (last) out[o + i * sd] = fx_to(R, em + 1 + Tab::gD);
+        else A[o + i * sd] = R;
+      }
+    }
+    first = false;
+    __syncthreads();
+  }
+}
+
+// dst_l = D_l src (the transposed derivative tables), l = 0..2: dst [3][5][nQ]
+template <int n>
+__device__ __forceinline__ void fx_grad(const double* src, double* dst) {
+  constexpr int n2 = n * n, nQ = n2 * n;
+  using Tab = FxTab<n>;
+  for (int t0 = threadIdx.x; t0 < 15 * n2; t0 += blockDim.x) {
+    const int l = t0 / (5 * n2), r = t0 - l * 5 * n2, v = r / n2;
+    int st, sd, fp;
+    fx_line_of<n>(l, r - v * n2, st, sd, fp);
+    const double* s = src + v * nQ + st;
+    double x[n];
+#pragma unroll
+    for (int m = 0; m < n; ++m) x[m] = s[m * sd];
+    FxD d[n];
+    const int eb = fx_line<n>(x, d) + 1 + Tab::gD;
+    double* o = dst + (5 * l + v) * nQ + st;
+#pragma unroll
+    for (int i = 0; i < n; ++i) o[i * sd] = fx_to(fx_dot<n>(d, [&](int m) { return Tab::D(m, i); }), eb);
+  }
+  __syncthreads();
+}
+
+// dst = D_l src along one direction
+template <int n>
+__device__ __forceinline__ void fx_grad1(int l, const double* src, double* dst) {
+  constexpr int n2 = n * n, nQ = n2 * n;
+  using Tab = FxTab<n>;
+  for (int t0 = threadIdx.x; t0 < 5 * n2; t0 += blockDim.x) {
+    const int v = t0 / n2;
+    int st, sd, fp;
+    fx_line_of<n>(l, t0 - v * n2, st, sd, fp);
+    const double* s = src + v * nQ + st;
+    double x[n];
+#pragma unroll
+    for (int m = 0; m < n; ++m) x[m] = s[m * sd];
+    FxD d[n];
+    const int eb = fx_line<n>(x, d) + 1 + Tab::gD;
+    double* o = dst + v * nQ + st;
+#pragma unroll
+    for (int i = 0; i < n; ++i) o[i * sd] = fx_to(fx_dot<n>(d, [&](int m) { return Tab::D(m, i); }), eb);
+  }
+  __syncthreads();
+}
+
+// buf += sum_f E_f^T (+-F_f): buf [5][nQ] doubles in place, F [nf][5][n^2]
+// doubles (both shared); neg 0x80000000 subtracts.  m: this lane's maxima of
+// the high words of buf and F (any partition of them over the lanes); the
+// words fx_slots() + 5 are clear, with a barrier since.
+template <int n>
+__device__ __forceinline__ void fx_lift(const TypeTab& T, double* buf, const double* F, unsigned neg,
+                                        const unsigned* m) {
+  constexpr int n2 = n * n, nQ = n2 * n;
+  using Tab = FxTab<n>;
+  unsigned* sx = fx_slots() + 5;
+  fx_flush_max(m, sx);
+  __syncthreads();
+  long long* A = reinterpret_cast<long long*>(buf);
+#pragma unroll 1
+  for (int l = 2; l >= 0; --l) {
+    const int lf0 = T.face_of[2 * l], lf1 = T.face_of[2 * l + 1];
+    for (int t0 = threadIdx.x; t0 < 5 * n2; t0 += blockDim.x) {
+      const int v = t0 / n2;
+      int st, sd, fp;
+      fx_line_of<n>(l, t0 - v * n2, st, sd, fp);
+      const int em = fx_em(sx[v]);
+      FxD d[2];
+      d[0] = d[1] = FxD{0, 0};
+      if (lf0 >= 0) d[0] = fx_split(fx_from(F[(lf0 * 5 + v) * n2 + fp], em, neg), 0);
+      if (lf1 >= 0) d[1] = fx_split(fx_from(F[(lf1 * 5 + v) * n2 + fp], em, neg), 0);
+      const int o = v * nQ + st;
+#pragma unroll
+      for (int i = 0; i < n; ++i) {
+        long long R = l == 2 ? fx_from(buf[o + i * sd], em + kFxGE) : A[o + i * sd];
+        R += fx_dot<2>(d, [&](int e) { return Tab::E(e, i); });
+        if (l == 0) buf[o + i * sd] = fx_to(R, em + 1 + kFxGE);
+        else A[o + i * sd] = R;
+      }
+    }
+    __syncthreads();
+  }
+}
+
+}  // namespace
+}  // namespace dgk

@@ -446,6 +446,41 @@ int Tables::add(int type, int N, std::string* err) {
         dput(d.tri ? w[ia] * w[ib] * 0.5 * (1 - be) : w[ia] * w[ib]);
       }
   }
+  // fixed-point copies of B and C for the integer contractions (dg_fixed.cuh).
+  // The factors of one mode reach 2^7 towards the degenerate edge while the
+  // low modes' stay near 1: every mode's row is scaled by a power of two to at
+  // most 1 (col_s, mode_s; the kernels apply it to the exponent of the mode's
+  // value), so that a sum over modes keeps the bits of its large terms.
+  fpool.resize(dpool.size(), dgk::FixPair{0, 0});
+  auto split = [](double c, int g) {
+    const int64_t C = (int64_t)std::nearbyint(std::ldexp(c, 62 - g));
+    const int64_t h = (C + ((int64_t)1 << 30)) >> 31;
+    return dgk::FixPair{(int)h, (int)(C - h * ((int64_t)1 << 31))};
+  };
+  auto balanced = [&](int off) {
+    double m = 0.0;
+    for (int k = 0; k < n; ++k) m = std::max(m, std::fabs(dpool[off + k]));
+    int e = 0;
+    while (m > std::ldexp(1.0, e)) ++e;
+    while (e > -60 && m > 0.0 && m <= std::ldexp(1.0, e - 1)) --e;
+    for (int k = 0; k < n; ++k) fpool[off + k] = split(std::ldexp(dpool[off + k], -e), 3);   // rows and columns: at most 7 terms < 2^3
+    return e;
+  };
+  t.col_s = ialloc(t.ncols);
+  t.mode_s = ialloc(t.nM);
+  for (int p = 0; p < n; ++p)
+    for (int q = 0; q < ipool[t.p_blen + p]; ++q)
+      ipool[t.col_s + ipool[t.p_cbase + p] + q] = balanced(t.B + ipool[t.p_boff + p] + q * n);
+  for (int col = 0; col < t.ncols; ++col)
+    for (int r = 0; r < ipool[t.col_len + col]; ++r)
+      ipool[t.mode_s + ipool[t.col_moff + col] + r] = balanced(t.C + ipool[t.col_coff + col] + r * n);
+  for (int i = 0; i < 2 * n; ++i) fpool[t.ext + i] = split(dpool[t.ext + i], 3);   // kFxGE
+  for (int k = 0; k < 6; ++k) t.face_of[k] = -1;
+  for (int lf = 0; lf < t.nfaces; ++lf) {
+    const FaceDesc d = t.faces[lf];
+    if (d.alpha > d.beta) { *err = "internal: face coordinates out of order"; return -1; }
+    t.face_of[2 * d.fixed + d.end] = lf;
+  }
   tabs.push_back(t);
   return (int)tabs.size() - 1;
 }

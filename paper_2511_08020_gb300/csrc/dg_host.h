@@ -20,6 +20,7 @@ void lagrange_values(const double* nodes, int n, double x, double* out);
 struct Tables {
   std::vector<double> dpool;
   std::vector<int> ipool;
+  std::vector<dgk::FixPair> fpool;   // fixed-point copies of the B and C tables, at their dpool offsets
   std::vector<dgk::TypeTab> tabs;
   int find(int type, int N) const;
   // returns table index or -1 with *err set

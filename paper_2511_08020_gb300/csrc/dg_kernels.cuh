@@ -43,6 +43,7 @@ enum ElemMode : int {
 struct Ctx {
   const double* dpool;
   const int* ipool;
+  const int2* fpool;           // fixed-point B and C tables (FixPair), at the dpool offsets
   const TypeTab* tabs;
   const int* slot_tab;
   const int8_t* slot_type;
@@ -67,6 +68,7 @@ struct Ctx {
   int flux;                    // 0 LF, 1 Roe, 2 entropy-conservative (Chandrashekar F#.n, no dissipation)
   int split;                   // 1: hexahedra evaluate the entropy-stable split form of the volume term
   int nQmax;
+  unsigned nmask;              // bit n: the launch covers elements with n points per direction
   // Navier-Stokes (BR1) state; ns == 0 for the Euler equations
   int ns;
   double mu, kappa;            // viscosity, heat conductivity mu gamma / ((gamma - 1) Pr)
@@ -152,7 +154,6 @@ void launch_faces(const Ctx& c, int64_t nblocks, int n, cudaStream_t st);
 // Navier-Stokes face phases: kind 0 = BR1 lifting values (T -> L), kind 1 =
 // inviscid + central viscous flux (T, Vt -> T).
 void launch_faces_ns(const Ctx& c, int64_t nblocks, int n, int kind, cudaStream_t st);
-int element_smem_bytes_ns(int nQmax);
 // phase 0: adjoint phase A (Euler), 2: phase C; Navier-Stokes adds 10: phase A
 // (inviscid + viscous flux transposes), 11: phase B (lifting transpose).
 void launch_vjp(const Ctx& c, int phase, const VjpArgs& va, int64_t nelem, int warps_per_block, cudaStream_t st);
@@ -173,10 +174,6 @@ void launch_halo_copy(const double* src, double* dst, const int64_t* off, int64_
                       cudaStream_t st, int mult = 1);
 void rk_params_node(cudaKernelNodeParams* p, void** args);
 bool is_rk_params_kernel(const void* func);
-int element_smem_bytes(int nQmax, int warps_per_block);
-// shared memory of an element launch: element_smem_bytes, or the split form's
-// larger workspace when c.split is set
-int element_launch_smem_bytes(int nQmax, int warps_per_block, bool split);
 int face_block_threads(int n);
 // curved: the mesh holds curved elements (occupancy of the kernel variants that handle them)
 cudaError_t element_kernel_attributes(int nQmax, int warps_per_block, int* blocks_per_sm, bool curved = false,
@@ -205,5 +202,22 @@ cudaError_t launch_moving_mass(const Ctx& c, const int64_t* list, int64_t n_slot
                                const double* x0, const double* tau, int weight, int max_nM, int max_nQ, int grid,
                                cudaStream_t st, int nblk = 1, int64_t blk_stride = 0, float* fac_out = nullptr,
                                const float* fac_in = nullptr);
+
+
+cudaError_t face_kernel_attributes();
+
+// The element launches of one build of dg_element.cu (one number of points
+// per direction n, one part: pointers of the other parts are null); a launch
+// skips elements of another n.
+struct ElemOps {
+  void (*element)(const Ctx& c, int mode, const StageArgs& a, const Sched& s, bool balanced, int grid, int wpb,
+                  cudaStream_t st);
+  void (*vjp)(const Ctx& c, int phase, const VjpArgs& va, int64_t nelem, int wpb, cudaStream_t st);
+  cudaError_t (*mass)(const Ctx& c, const int64_t* list, int64_t n_slots, const double* in, double* out,
+                      const double* x0, const double* tau, int weight, int max_nM, int max_nQ, int grid,
+                      cudaStream_t st, int nblk, int64_t blk_stride, float* fac_out, const float* fac_in);
+  // shared-memory limits; resident blocks per SM of the part's main kernel
+  cudaError_t (*attributes)(int wpb, int* blocks_per_sm, bool curved, bool split);
+};
 
 }  // namespace dgk

@@ -5,7 +5,7 @@
 // point's area vector a quadratic.  These kernels evaluate the geometry of
 // the static curved path at a time t from those coefficients (the mass
 // matrix kernel of the stage solves sits with the element transforms it
-// uses, in dg_kernels.cu).
+// uses, in dg_element.cu).
 #include "dg_kernels.cuh"
 
 namespace dgk {
