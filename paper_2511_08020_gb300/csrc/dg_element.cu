@@ -6,6 +6,9 @@
 // solves (1), the adjoint phases (2).  See dg_kernels.cuh for the phase layout.
 #include <algorithm>
 
+#if DG_PART == 1
+#define DG_UNROLL 1
+#endif
 #include "dg_fixed.cuh"
 #include "dg_physics.cuh"
 
@@ -18,12 +21,19 @@ namespace dgk {
 namespace {
 
 constexpr int kn = DG_N, kn2 = kn * kn, knQ = kn2 * kn;
+// bufG of the Navier-Stokes volume phase: two blocks of [5][nQ], or the face
+// values of six faces
+constexpr int kNsG = 10 * knQ > 30 * kn2 ? 10 * knQ : 30 * kn2;
 
 // Kernel families: the phases of a stage, the Navier-Stokes volume phase, and
 // the one-shot maps (projection, evaluation, conversions, trace rebuilds).
 enum Family { kStage = 0, kNs = 1, kMisc = 2 };
 
-constexpr int kStageBlocks = kn <= 5 ? 6 : 5, kNsBlocks = kn <= 5 ? 5 : (kn == 6 ? 3 : 2);
+// Resident blocks per SM the registers are limited to.  The stage phases wait
+// for latencies (tables, barriers, dependent multiply-adds), so warps count for
+// more than a few spilled registers: 16^3 mixed N = 4, two steps, 5.83 / 5.63 /
+// 5.52 ms with 6 / 7 / 8 blocks; N = 5 and 6 are limited by shared memory.
+constexpr int kStageBlocks = kn <= 5 ? 8 : 5, kNsBlocks = kn <= 5 ? 6 : (kn == 6 ? 4 : 2);
 
 // ------------------------------------------------------------------ element phases
 //
@@ -68,7 +78,7 @@ __device__ __forceinline__ void modal_to_nodal(const Ctx& c, const TypeTab& T, c
 // What the nodal->modal pass does with r = M_ref^{-1} V^T bufA of a mode
 // (r = V^T bufA without the mass matrix when minv == false):
 //   kStore: out[v nM + m] = scale r_v
-//   kRk:    K <- a K + dt scale r (a == 0: K <- dt scale r), Q <- Q + b K,
+//   kRk:    K <- a K + scale r (a == 0: K <- scale r; scale includes dt), Q <- Q + b K,
 //           and the new Q is also written to sQ when sQ != nullptr.
 //   kAxpy:  out[v nM + m] += scale r_v
 struct Epilogue {
@@ -81,7 +91,7 @@ struct Epilogue {
   double* Qo;
   double* K;
   double* sQ;
-  double a, b, dt;
+  double a, b;
   // curved prism / pyramid: r = Md (V^T bufA) with the element's dense
   // inverse mass matrix Md [nM][nM] (symmetric) instead of minv and scale;
   // rbuf [5][nM] is shared scratch that no other argument aliases
@@ -107,7 +117,7 @@ __device__ __forceinline__ bool epilogue_mode(const Epilogue& ep, int nM, int mo
     for (int v = 0; v < 5; ++v) {
       const int idx = v * nM + mode;
       const double R = r[v];
-      const double k = (ep.a == 0.0) ? ep.dt * R : fma(ep.a, ep.K[idx], ep.dt * R);
+      const double k = (ep.a == 0.0) ? R : fma(ep.a, ep.K[idx], R);   // r carries dt
       const double qn = fma(ep.b, k, ep.Qi[idx]);
       ep.K[idx] = k;
       ep.Qo[idx] = qn;
@@ -121,7 +131,7 @@ __device__ __forceinline__ bool epilogue_mode(const Epilogue& ep, int nM, int mo
 // Applies `ep` to r = V^T h (doubles [5][nM], shared).  Returns true if a
 // non-finite state value was produced.
 template <bool DENSE>
-__device__ __forceinline__ bool finish_modal(const Ctx& c, const TypeTab& T, const double* r, int lane,
+__device__ __forceinline__ bool finish_modal(const Ctx& c, const TypeTab& T, double* r, int lane,
                                              const Epilogue& ep) {
   const int nM = T.nM;
   const double* dp = c.dpool;
@@ -138,16 +148,12 @@ __device__ __forceinline__ bool finish_modal(const Ctx& c, const TypeTab& T, con
   if (DENSE) {
     // dense inverse mass matrix of a curved element (Algorithm 1 with a
     // pointwise J): lanes run over output modes, so the column reads of the
-    // symmetric Md are coalesced and every load feeds 5 FMAs
-    for (int mode = lane; mode < nM; mode += blockDim.x) {
-      const double* Mc = ep.Md + mode;
-      double acc[5] = {0, 0, 0, 0, 0};
-#pragma unroll 4
-      for (int j = 0; j < nM; ++j) DG_FMA5(Mc[(size_t)j * nM], r + j, nM, acc);
+    // symmetric Md are coalesced and every load feeds 5 sums
+    fx_dense(ep.Md, r, nM, [&](int mode, double* acc) {
 #pragma unroll
       for (int v = 0; v < 5; ++v) acc[v] *= ep.scale;
       bad |= epilogue_mode(ep, nM, mode, acc);
-    }
+    });
   }
   __syncthreads();
   return bad;
@@ -205,19 +211,6 @@ __device__ __forceinline__ void write_traces(const Ctx& c, const TypeTab& T, int
                                              double* dst, unsigned neg = 0u, int ft_mult = 1, int64_t ft_add = 0) {
   const int64_t* ft = c.slot_ftoff + s * 6;
   write_traces_n<kn>(T, ft, src, dst, neg, ft_mult, ft_add);
-}
-
-// out = sum over the directions in `dirs` of D_l^T G_l (G at bufG, [3][5][nQ],
-// destroyed; out may be its first block when no direction below the last one
-// used reads it).  scanned: the largest high words of G are in fx_slots() + 10.
-template <int n>
-__device__ __forceinline__ void dsum_n(double* bufG, unsigned dirs, double* out, bool scanned) {
-  fx_dsum_body<n>(bufG, dirs, bufG + 10 * n * n * n, out, fx_slots() + 10, scanned);
-}
-
-__device__ __forceinline__ void derivative_sum(const TypeTab& T, double* bufG, unsigned dirs, double* out,
-                                               bool scanned) {
-  dsum_n<kn>(bufG, dirs, out, scanned);
 }
 
 // Structurally nonzero entries of d(a,b,c)_l / d(xi)_k per type: bit l*3+k.
@@ -522,7 +515,10 @@ __device__ __forceinline__ void element_forward_t(const Ctx& c, const TypeTab& T
   }
   fx_flush_max(mg, fx_slots() + 10);
   // H = sum_l D_l^T G_l (collocation derivative along each collapsed direction)
-  derivative_sum(T, bufG, 7u, c.H + c.slot_hoff[s], true);
+  // (the last direction's sums run in place of its own G)
+  __syncthreads();
+  fx_dsum<kn>([&](int l, int v, int q) { return bufG[(5 * l + v) * nQ + q]; },
+              [&](int v) { return fx_em(fx_slots()[10 + v]); }, 7u, bufG + 10 * nQ, c.H + c.slot_hoff[s]);
 }
 
 template <bool ANY, bool SPLIT>
@@ -622,17 +618,20 @@ __device__ __forceinline__ void lift_scaled_t(const Ctx& c, const TypeTab& T, in
 //   nodal  grad_d W = V G_d, and its traces on the own face points (Vt);
 // then the total flux F_e(U) - F_v(U, grad W) at the volume points and
 // H = sum_l D_l^T G_l(F) as in the Euler forward phase.
-// smem: bufU [5 nQ] | bufDW [3][5][nQ] | bufG [15 nQ] | bufA [5 nQ].
+// smem: bufA [5 nQ] | bufDW [3][5][nQ] | bufG [kNsG].  The products with the
+// metric are formed where a derivative pass reads them and the total flux
+// overwrites the gradient, so an element takes 30 nQ doubles (40 with buffers of
+// their own: fewer resident blocks, and the phase waits for latencies).
 template <bool CURVED>
 __device__ __forceinline__ void element_ns_volume_t(const Ctx& c, const TypeTab& T, int64_t s, double* smem, int lane) {
   constexpr int n = kn, nQ = knQ, n2 = kn2;
   // curved element: pointwise metric [9][nQ], J, 1/J, (prism, pyramid) dense M_e^{-1}
   const double* cblk = CURVED ? c.cpool + c.slot_coff[s] : nullptr;
   constexpr int nQm = knQ;
-  double* bufU = smem;
+  double* bufA = smem;
   double* bufDW = smem + 5 * nQm;
   double* bufG = smem + 20 * nQm;
-  double* bufA = smem + 35 * nQm;
+  const double* Un = c.Unod + c.slot_hoff[s];
   const double* dp = c.dpool;
   const double gm1 = c.gamma - 1.0;
   const ElemGeo& g = c.geo[s];
@@ -643,11 +642,6 @@ __device__ __forceinline__ void element_ns_volume_t(const Ctx& c, const TypeTab&
   // M(t)^{-1}; hexahedra run whole in phase 2
   const bool dense_split = CURVED && c.lift_phase != 0 && T.type != HEX;
   if (CURVED && c.lift_phase == 1 && !dense_split) return;
-  {
-    const double* Un = c.Unod + c.slot_hoff[s];
-    for (int w = lane; w < 5 * nQ; w += blockDim.x) bufU[w] = Un[w];
-  }
-  __syncthreads();
   if (dense_split && c.lift_phase == 2) {
     // the solved modal gradient of every direction: nodal values, traces
     for (int d = 0; d < 3; ++d) {
@@ -670,53 +664,49 @@ __device__ __forceinline__ void element_ns_volume_t(const Ctx& c, const TypeTab&
   for (int q = lane; q < nQ; q += blockDim.x) {
     double U[5], W[5];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) U[v] = bufU[v * nQ + q];
+    for (int v = 0; v < 5; ++v) U[v] = Un[v * nQ + q];
     primitive(U, gm1, W);
 #pragma unroll
     for (int v = 0; v < 5; ++v) bufA[v * nQ + q] = W[v];
   }
-  __syncthreads();
-  if (CURVED) {
-    // pointwise metric: Hd = sum_l D_l^T (M_q[l][d] W), one full set of
-    // directional passes per direction d
-    for (int d = 0; d < 3; ++d) {
-      for (int q = lane; q < nQ; q += blockDim.x) {
-#pragma unroll
+  const unsigned nz = kMetricMask[T.type];
+  int* es = reinterpret_cast<int*>(fx_slots()) + 10;
+#pragma unroll 1
+  for (int k = 0; k < 3; ++k) {
+    // affine: P_k; a curved element takes one full set of directional passes
+    // per direction with its pointwise metric, H_d = sum_l D_l^T (M_q[l][d] W)
+    const unsigned dirs = CURVED ? 7u : ((nz >> k) & 1u) | (((nz >> (3 + k)) & 1u) << 1) | (((nz >> (6 + k)) & 1u) << 2);
+    auto metric = [&](int l, int q) {
+      return CURVED ? cblk[(l * 3 + k) * nQ + q] : __ldg(dp + T.wA + q * 9 + l * 3 + k);
+    };
+    if (lane < 5) es[lane] = -4096;
+    __syncthreads();
+    {
+      int m[5] = {-4096, -4096, -4096, -4096, -4096};
+      for (int q = lane; q < nQ; q += blockDim.x)
         for (int l = 0; l < 3; ++l) {
-          const double f = cblk[(l * 3 + d) * nQ + q];
+          if (!((dirs >> l) & 1u)) continue;
+          const double f = metric(l, q);
 #pragma unroll
-          for (int v = 0; v < 5; ++v) bufG[(l * 5 + v) * nQ + q] = f * bufA[v * nQ + q];
+          for (int v = 0; v < 5; ++v) m[v] = max(m[v], fx_em_product(f, fx_hi(bufA[v * nQ + q])));
+        }
+      fx_flush_max(m, es);
+    }
+    __syncthreads();
+    fx_dsum<kn>([&](int l, int v, int q) { return metric(l, q) * bufA[v * nQ + q]; }, [&](int v) { return es[v]; }, dirs,
+                bufG + 5 * nQ, CURVED ? bufDW + k * 5 * nQ : bufG);
+    if (!CURVED) {
+      for (int w = lane; w < 5 * nQ; w += blockDim.x) {
+        const double p = bufG[w];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          double* Hd = bufDW + d * 5 * nQ + w;
+          const double jkd = Jg[k * 3 + d];
+          *Hd = k == 0 ? jkd * p : fma(jkd, p, *Hd);
         }
       }
       __syncthreads();
-      derivative_sum(T, bufG, 7u, bufDW + d * 5 * nQ, false);
     }
-  }
-  const unsigned nz = kMetricMask[T.type];
-  for (int kr = 0; kr < (CURVED ? 0 : 3); ++kr) {
-    const unsigned dirs = ((nz >> kr) & 1u) | (((nz >> (3 + kr)) & 1u) << 1) | (((nz >> (6 + kr)) & 1u) << 2);
-    for (int q = lane; q < nQ; q += blockDim.x) {
-      const double* wa = dp + T.wA + q * 9;
-#pragma unroll
-      for (int l = 0; l < 3; ++l) {
-        if (!((nz >> (l * 3 + kr)) & 1u)) continue;
-        const double f = wa[l * 3 + kr];
-#pragma unroll
-        for (int v = 0; v < 5; ++v) bufG[(l * 5 + v) * nQ + q] = f * bufA[v * nQ + q];
-      }
-    }
-    __syncthreads();
-    derivative_sum(T, bufG, dirs, bufG, false);   // P_k
-    for (int w = lane; w < 5 * nQ; w += blockDim.x) {
-      const double p = bufG[w];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        double* Hd = bufDW + d * 5 * nQ + w;
-        const double jkd = Jg[kr * 3 + d];
-        *Hd = kr == 0 ? jkd * p : fma(jkd, p, *Hd);
-      }
-    }
-    __syncthreads();
   }
 #pragma unroll 1
   for (int d = 0; d < 3; ++d) {
@@ -739,7 +729,6 @@ __device__ __forceinline__ void element_ns_volume_t(const Ctx& c, const TypeTab&
     } else {
       // r = V^T (Hd - sum_f n_d(f) E_f^T L_f), then the projection
       const int64_t* ft = c.slot_ftoff + s * 6;
-      double* r = CURVED && !dense_split ? bufG + 10 * nQ : bufA;
       fx_lift_to_modal<kn>(
           c, T, [&](int o) { return dW[o]; },
           [&](int lf, int v, int p) {
@@ -747,18 +736,18 @@ __device__ __forceinline__ void element_ns_volume_t(const Ctx& c, const TypeTab&
             const double nd = CURVED ? c.snrm[3 * (t / 5) + d * n2 + p] : c.fnrm[(s * 6 + lf) * 3 + d];
             return nd * c.L[t + v * n2 + p];
           },
-          0x80000000u, bufA, bufG, r);
+          0x80000000u, bufA, bufG, bufA);
       if (dense_split) {
         // phase 1: r_d = -V^T (lifting terms); M(t)^{-1} r_d is solved outside
         Epilogue ep{Epilogue::kStore, false, -1.0, c.lift + (int64_t)d * c.lift_stride + c.slot_qoff[s], nullptr,
-                    nullptr, nullptr, nullptr, 0.0, 0.0, 0.0};
-        finish_modal<false>(c, T, r, lane, ep);
+                    nullptr, nullptr, nullptr, 0.0, 0.0};
+        finish_modal<false>(c, T, bufA, lane, ep);
         continue;
       }
       double* sG = bufG + 5 * nQ;
-      Epilogue ep{Epilogue::kStore, true, CURVED ? -1.0 : -g.invJ, sG, nullptr, nullptr, nullptr, nullptr, 0.0, 0.0, 0.0};
+      Epilogue ep{Epilogue::kStore, true, CURVED ? -1.0 : -g.invJ, sG, nullptr, nullptr, nullptr, nullptr, 0.0, 0.0};
       if (CURVED) ep.Md = cblk + 11 * nQ;
-      finish_modal<CURVED>(c, T, r, lane, ep);
+      finish_modal<CURVED>(c, T, bufA, lane, ep);
       fx_to_nodal<kn, true>(c, T, sG, dW, bufG, [&](int lf, int v, int p, double x) {
         c.Vt[3 * __ldg(ft + lf) + (d * 5 + v) * n2 + p] = x;
       });
@@ -772,10 +761,18 @@ __device__ __forceinline__ void element_ns_volume_t(const Ctx& c, const TypeTab&
   if (dense_split) return;   // phase 1 ends with the lifting residuals
   }
   // total contravariant flux G_l = sum_d M[l][d] (F_e - F_v)_d
+  // (in place of the point's gradient)
+  fx_clear(fx_slots() + 10, 5);
+  __syncthreads();
+  unsigned mg[5] = {0u, 0u, 0u, 0u, 0u};   // largest high words of G per variable
+  auto put = [&](double* G, int v, double x) {
+    G[v * nQ] = x;
+    mg[v] = max(mg[v], fx_hi(x));
+  };
   for (int q = lane; q < nQ; q += blockDim.x) {
     double U[5], W[5], gr[15];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) U[v] = bufU[v * nQ + q];
+    for (int v = 0; v < 5; ++v) U[v] = Un[v * nQ + q];
 #pragma unroll
     for (int t = 0; t < 15; ++t) gr[t] = bufDW[t * nQ + q];
     primitive(U, gm1, W);
@@ -799,28 +796,30 @@ __device__ __forceinline__ void element_ns_volume_t(const Ctx& c, const TypeTab&
       for (int l = 0; l < 3; ++l) {
         const double Vl = M[l][0] * u + M[l][1] * v + M[l][2] * w;
         const double Rl = Vl - (M[l][0] * x0 + M[l][1] * x1 + M[l][2] * x2);
-        double* G = bufG + l * 5 * nQ + q;
-        G[0] = Rl * U[0];
-        G[nQ] = Rl * U[1] + p * M[l][0] - (M[l][0] * Fv[0][1] + M[l][1] * Fv[1][1] + M[l][2] * Fv[2][1]);
-        G[2 * nQ] = Rl * U[2] + p * M[l][1] - (M[l][0] * Fv[0][2] + M[l][1] * Fv[1][2] + M[l][2] * Fv[2][2]);
-        G[3 * nQ] = Rl * U[3] + p * M[l][2] - (M[l][0] * Fv[0][3] + M[l][1] * Fv[1][3] + M[l][2] * Fv[2][3]);
-        G[4 * nQ] = Rl * U[4] + Vl * p - (M[l][0] * Fv[0][4] + M[l][1] * Fv[1][4] + M[l][2] * Fv[2][4]);
+        double* G = bufDW + l * 5 * nQ + q;
+        put(G, 0, Rl * U[0]);
+        put(G, 1, Rl * U[1] + p * M[l][0] - (M[l][0] * Fv[0][1] + M[l][1] * Fv[1][1] + M[l][2] * Fv[2][1]));
+        put(G, 2, Rl * U[2] + p * M[l][1] - (M[l][0] * Fv[0][2] + M[l][1] * Fv[1][2] + M[l][2] * Fv[2][2]));
+        put(G, 3, Rl * U[3] + p * M[l][2] - (M[l][0] * Fv[0][3] + M[l][1] * Fv[1][3] + M[l][2] * Fv[2][3]));
+        put(G, 4, Rl * U[4] + Vl * p - (M[l][0] * Fv[0][4] + M[l][1] * Fv[1][4] + M[l][2] * Fv[2][4]));
       }
       continue;
     }
 #pragma unroll
     for (int l = 0; l < 3; ++l) {
       double Vl = M[l][0] * u + M[l][1] * v + M[l][2] * w;
-      double* G = bufG + l * 5 * nQ + q;
-      G[0] = Vl * U[0];
-      G[nQ] = Vl * U[1] + p * M[l][0] - (M[l][0] * Fv[0][1] + M[l][1] * Fv[1][1] + M[l][2] * Fv[2][1]);
-      G[2 * nQ] = Vl * U[2] + p * M[l][1] - (M[l][0] * Fv[0][2] + M[l][1] * Fv[1][2] + M[l][2] * Fv[2][2]);
-      G[3 * nQ] = Vl * U[3] + p * M[l][2] - (M[l][0] * Fv[0][3] + M[l][1] * Fv[1][3] + M[l][2] * Fv[2][3]);
-      G[4 * nQ] = Vl * Ep - (M[l][0] * Fv[0][4] + M[l][1] * Fv[1][4] + M[l][2] * Fv[2][4]);
+      double* G = bufDW + l * 5 * nQ + q;
+      put(G, 0, Vl * U[0]);
+      put(G, 1, Vl * U[1] + p * M[l][0] - (M[l][0] * Fv[0][1] + M[l][1] * Fv[1][1] + M[l][2] * Fv[2][1]));
+      put(G, 2, Vl * U[2] + p * M[l][1] - (M[l][0] * Fv[0][2] + M[l][1] * Fv[1][2] + M[l][2] * Fv[2][2]));
+      put(G, 3, Vl * U[3] + p * M[l][2] - (M[l][0] * Fv[0][3] + M[l][1] * Fv[1][3] + M[l][2] * Fv[2][3]));
+      put(G, 4, Vl * Ep - (M[l][0] * Fv[0][4] + M[l][1] * Fv[1][4] + M[l][2] * Fv[2][4]));
     }
   }
+  fx_flush_max(mg, fx_slots() + 10);
   __syncthreads();
-  derivative_sum(T, bufG, 7u, c.H + c.slot_hoff[s], false);
+  fx_dsum<kn>([&](int l, int v, int q) { return bufDW[(5 * l + v) * nQ + q]; },
+              [&](int v) { return fx_em(fx_slots()[10 + v]); }, 7u, bufG, c.H + c.slot_hoff[s]);
 }
 
 template <bool ANY>
@@ -830,7 +829,7 @@ __device__ __forceinline__ void element_ns_volume(const Ctx& c, const TypeTab& T
 }
 
 // One element at slot s.  smem per block: bufA [5 nQ], bufG [15 nQ]
-// (40 nQ for the Navier-Stokes volume phase).
+// (30 nQ for the Navier-Stokes volume phase).
 template <int FAM, bool ANY, bool SPLIT>
 __device__ __forceinline__ void process_element(const Ctx& c, int mode, const StageArgs& io, int64_t s, double* bufA,
                                                 double* bufG, int lane) {
@@ -838,11 +837,11 @@ __device__ __forceinline__ void process_element(const Ctx& c, int mode, const St
   constexpr int nQ = knQ;
   const int nM = T.nM;
   const int64_t qoff = c.slot_qoff[s];
-  if (FAM == kNs) {
+  if constexpr (FAM == kNs) {
     element_ns_volume<ANY>(c, T, s, bufA, lane);
     return;
   }
-  if (FAM == kMisc && mode == kGather) {
+  if constexpr (FAM == kMisc) if (mode == kGather) {
     // hexahedra only: caller modal coefficients Q -> storage s = W^{1/2} V Q
     const double* Q = io.Qin + c.elem_qoff[c.elem_of_slot[s]];
     for (int w = lane; w < 5 * nM; w += blockDim.x) bufG[w] = Q[w];
@@ -854,26 +853,26 @@ __device__ __forceinline__ void process_element(const Ctx& c, int mode, const St
     __syncthreads();
     return;
   }
-  if (FAM == kMisc && mode == kScatter) {
+  if constexpr (FAM == kMisc) if (mode == kScatter) {
     // hexahedra only: storage s -> caller modal coefficients V^T W^{1/2} s
     const double* S = io.Qin + qoff;
     const double* sq = c.dpool + T.sqw;
     for (int w = lane; w < 5 * nQ; w += blockDim.x) bufA[w] = S[w] * sq[w % nQ];
     __syncthreads();
     Epilogue ep{Epilogue::kStore, false, 1.0, io.Qout + c.elem_qoff[c.elem_of_slot[s]], nullptr, nullptr, nullptr,
-                nullptr, 0.0, 0.0, 0.0};
+                nullptr, 0.0, 0.0};
     ep.modal = true;
     nodal_to_modal_t<false>(c, T, bufA, bufG, lane, ep);
     return;
   }
-  if (FAM == kStage && mode == kFwd) {
+  if constexpr (FAM == kStage) if (mode == kFwd) {
     const double* Q = io.Qin + qoff;
     for (int w = lane; w < 5 * nM; w += blockDim.x) bufG[w] = Q[w];
     __syncthreads();
     element_forward<ANY, SPLIT>(c, T, s, bufA, bufG, lane);
     return;
   }
-  if (FAM == kMisc && mode == kTraces) {
+  if constexpr (FAM == kMisc) if (mode == kTraces) {
     // the stage's face traces rebuilt from its kept nodal state (and the
     // gradient traces from its kept nodal gradient) by the same trace
     // writes as the forward phases: bitwise the values they wrote
@@ -893,7 +892,7 @@ __device__ __forceinline__ void process_element(const Ctx& c, int mode, const St
     __syncthreads();
     return;
   }
-  if (FAM == kMisc && mode == kEval) {
+  if constexpr (FAM == kMisc) if (mode == kEval) {
     const double* Q = io.Qin + qoff;
     for (int w = lane; w < 5 * nM; w += blockDim.x) bufG[w] = Q[w];
     __syncthreads();
@@ -913,7 +912,7 @@ __device__ __forceinline__ void process_element(const Ctx& c, int mode, const St
   // the mass-weighted state; the mass matrix is solved separately)
   const bool moving = ANY && c.mpool != nullptr;
   const bool dense = cblk && T.type != HEX && (!moving || FAM == kMisc);
-  if (FAM == kMisc && mode == kLoad) {
+  if constexpr (FAM == kMisc) if (mode == kLoad) {
     // b = V^T W J q: pointwise J_q (curved) or the element's constant J
     const int64_t e = c.elem_of_slot[s];
     const double* vals = io.Qin + c.elem_voff[e];
@@ -926,11 +925,11 @@ __device__ __forceinline__ void process_element(const Ctx& c, int mode, const St
     }
     __syncthreads();
     Epilogue ep{Epilogue::kStore, false, cblk ? 1.0 : 1.0 / c.geo[s].invJ, io.Qout + qoff, nullptr, nullptr, nullptr,
-                nullptr, 0.0, 0.0, 0.0};
+                nullptr, 0.0, 0.0};
     nodal_to_modal<false>(c, T, bufA, bufG, lane, ep);
     return;
   }
-  if (FAM == kMisc && mode == kProject) {
+  if constexpr (FAM == kMisc) if (mode == kProject) {
     const int64_t e = c.elem_of_slot[s];
     const double* vals = io.Qin + c.elem_voff[e];
     const double* W = c.dpool + T.W;
@@ -941,7 +940,7 @@ __device__ __forceinline__ void process_element(const Ctx& c, int mode, const St
       for (int w = lane; w < 5 * nQ; w += blockDim.x) bufA[w] = W[w % nQ] * vals[w];
     }
     __syncthreads();
-    Epilogue ep{Epilogue::kStore, true, 1.0, io.Qout + qoff, nullptr, nullptr, nullptr, nullptr, 0.0, 0.0, 0.0};
+    Epilogue ep{Epilogue::kStore, true, 1.0, io.Qout + qoff, nullptr, nullptr, nullptr, nullptr, 0.0, 0.0};
     if (dense) {
       ep.Md = cblk + 11 * nQ;
       ep.rbuf = bufG + 5 * nQ;
@@ -949,20 +948,21 @@ __device__ __forceinline__ void process_element(const Ctx& c, int mode, const St
     nodal_to_modal<ANY>(c, T, bufA, bufG, lane, ep);
     return;
   }
-  if (FAM != kStage) return;
-  const double* pscale = (cblk && T.type == HEX && !moving) ? cblk + 10 * nQ : nullptr;
-  const double invJ = cblk ? 1.0 : c.geo[s].invJ;
-  // one epilogue for both kinds of step, so that the backward code exists once
-  const bool rhs = mode == kBwdRhs;
-  Epilogue ep{rhs ? Epilogue::kStore : Epilogue::kRk, !moving, invJ, rhs ? io.Qout + qoff : nullptr, io.Qin + qoff,
-              io.Qout + qoff, io.K + qoff, mode == kBwdRkFwd ? bufG : nullptr, io.a, io.b, io.dt};
-  if (dense) {
-    ep.Md = cblk + 11 * nQ;
-    ep.rbuf = bufG + 5 * nQ;
+  if constexpr (FAM == kStage) {
+    const double* pscale = (cblk && T.type == HEX && !moving) ? cblk + 10 * nQ : nullptr;
+    const double invJ = cblk ? 1.0 : c.geo[s].invJ;
+    // one epilogue for both kinds of step, so that the backward code exists once
+    const bool rhs = mode == kBwdRhs;
+    Epilogue ep{rhs ? Epilogue::kStore : Epilogue::kRk, !moving, rhs ? invJ : invJ * io.dt, rhs ? io.Qout + qoff : nullptr, io.Qin + qoff,
+                io.Qout + qoff, io.K + qoff, mode == kBwdRkFwd ? bufG : nullptr, io.a, io.b};
+    if (dense) {
+      ep.Md = cblk + 11 * nQ;
+      ep.rbuf = bufG + 5 * nQ;
+    }
+    const bool bad = __syncthreads_or(element_backward<ANY>(c, T, s, bufA, bufG, lane, c.T, 0x80000000u, pscale, ep));
+    if (bad && lane == 0) atomicOr(c.status, 1u);
+    if (mode == kBwdRkFwd) element_forward<ANY, SPLIT>(c, T, s, bufA, bufG, lane);
   }
-  const bool bad = __syncthreads_or(element_backward<ANY>(c, T, s, bufA, bufG, lane, c.T, 0x80000000u, pscale, ep));
-  if (bad && lane == 0) atomicOr(c.status, 1u);
-  if (mode == kBwdRkFwd) element_forward<ANY, SPLIT>(c, T, s, bufA, bufG, lane);
 }
 
 // ------------------------------------------------------------------ adjoint element phases
@@ -1021,13 +1021,10 @@ __device__ __forceinline__ void element_vjp_a_t(const Ctx& c, const VjpArgs& va,
   __syncthreads();
   if (dense) {
     const double* Md = cblk + 11 * nQ;
-    for (int m = lane; m < nM; m += blockDim.x) {
-      double acc[5] = {0, 0, 0, 0, 0};
-#pragma unroll 4
-      for (int j = 0; j < nM; ++j) DG_FMA5(Md[(size_t)j * nM + m], bufC + j, nM, acc);
+    fx_dense(Md, bufC, nM, [&](int m, double* acc) {
 #pragma unroll
       for (int v = 0; v < 5; ++v) bufG[v * nM + m] = acc[v];
-    }
+    });
     __syncthreads();
   }
   modal_to_nodal(c, T, bufG, bufC, bufG + 5 * nQm, lane);  // Ybar in bufC
@@ -1086,7 +1083,7 @@ __device__ __forceinline__ void element_vjp_c(const Ctx& c, const VjpArgs& va, i
                                            int lane) {
   const TypeTab& T = c.tabs[c.slot_tab[s]];
   Epilogue ep{va.rk ? Epilogue::kAxpy : Epilogue::kStore, false, va.rk ? va.dt : 1.0, va.Qbar + c.slot_qoff[s],
-              nullptr, nullptr, nullptr, nullptr, 0.0, 0.0, 0.0};
+              nullptr, nullptr, nullptr, nullptr, 0.0, 0.0};
   element_backward<false>(c, T, s, bufA, bufG, lane, c.Tv, 0u, nullptr, ep);
 }
 
@@ -1156,13 +1153,10 @@ __device__ __forceinline__ void element_vjp_a_ns_t(const Ctx& c, const VjpArgs& 
   __syncthreads();
   if (dense) {
     const double* Md = cblk + 11 * nQ;
-    for (int m = lane; m < nM; m += blockDim.x) {
-      double acc[5] = {0, 0, 0, 0, 0};
-#pragma unroll 4
-      for (int j = 0; j < nM; ++j) DG_FMA5(Md[(size_t)j * nM + m], bufY + j, nM, acc);
+    fx_dense(Md, bufY, nM, [&](int m, double* acc) {
 #pragma unroll
       for (int v = 0; v < 5; ++v) bufS[v * nM + m] = acc[v];
-    }
+    });
     __syncthreads();
   }
   modal_to_nodal(c, T, bufS, bufY, bufG, lane);
@@ -1278,7 +1272,7 @@ __device__ __forceinline__ void element_vjp_b_ns_t(const Ctx& c, int64_t s, doub
       }
       __syncthreads();
     } else {
-      Epilogue ep{Epilogue::kStore, true, CURVED ? -1.0 : -g.invJ, bufX, nullptr, nullptr, nullptr, nullptr, 0.0, 0.0, 0.0};
+      Epilogue ep{Epilogue::kStore, true, CURVED ? -1.0 : -g.invJ, bufX, nullptr, nullptr, nullptr, nullptr, 0.0, 0.0};
       if (CURVED) {
         ep.Md = cblk + 11 * nQ;        // symmetric: its own transpose
         ep.rbuf = smem + 15 * nQm;
@@ -1490,7 +1484,7 @@ __device__ void mass_product(const Ctx& c, const TypeTab& T, const double* x, co
   modal_to_nodal_passes(c, T, x, bufA, bufB);
   for (int w = tid; w < 5 * nQ; w += blockDim.x) bufA[w] *= wJ[w % nQ];
   __syncthreads();
-  Epilogue ep{Epilogue::kStore, false, 1.0, r, nullptr, nullptr, nullptr, nullptr, 0.0, 0.0, 0.0};
+  Epilogue ep{Epilogue::kStore, false, 1.0, r, nullptr, nullptr, nullptr, nullptr, 0.0, 0.0};
   nodal_to_modal_t<false>(c, T, bufA, bufB, tid, ep);
   if (b) {
     for (int w = tid; w < 5 * nM; w += blockDim.x) r[w] = b[w] - r[w];
@@ -1796,7 +1790,7 @@ cudaError_t set_smem(K kernel, int bytes) {
 }
 
 constexpr int kD = (int)sizeof(double);
-constexpr int kStageBytes = 20 * knQ * kD, kNsBytes = 40 * knQ * kD;
+constexpr int kStageBytes = 20 * knQ * kD, kNsBytes = (20 * knQ + kNsG) * kD;
 // the split form's workspace: bufA [5 nQ] + two-point quantities [kTP][nQ] +
 // face states [kTP][6 n^2] + one direction's pair fluxes [n^2][n(n-1)/2][5]
 // and face-state fluxes [n^2][2 n][5]

@@ -30,9 +30,17 @@
 // from the table pool.
 #pragma once
 #include "dg_kernels.cuh"
+// Unrolling of the loops over a line's results.  A kernel that runs every pass
+// once per element keeps them unrolled; the Navier-Stokes volume phase, whose
+// code is long, is faster rolled (fewer instruction-cache misses: the viscous
+// 20^3 step 21.09 -> 20.07 ms; the Euler step 5.52 unrolled, 5.57 rolled).
+#ifndef DG_UNROLL
+#define DG_UNROLL 8
+#endif
 
 namespace dgk {
 namespace {
+constexpr int kUnroll = DG_UNROLL;
 
 // Tables per n: coefficient c is stored as round(c 2^(62 - g)) =
 // x 2^31 + y with -2^30 <= y < 2^30; g bounds every row (and column) sum of
@@ -220,6 +228,7 @@ __device__ __forceinline__ FxD fx_split(long long D, int k) {
   FxD f;
   f.h = (int)__funnelshift_r(lo, hi, 31 - k);
   f.l = (int)((lo << k) & 0x7fffffffu);
+  asm("" : "+r"(f.l));   // see fx_madw
   return f;
 }
 
@@ -272,24 +281,24 @@ __device__ __forceinline__ unsigned fx_mag(long long R) {
   return (unsigned)(h ^ (h >> 31));
 }
 
-// a b + c, one instruction (written out: the C++ expression on operands that
-// the compiler has already widened becomes a three-instruction 64-bit product)
-__device__ __forceinline__ long long fx_madw(int a, int b, long long c) {
-  long long r;
-  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
-  return r;
-}
+// a b + c: one IMAD.WIDE as long as the compiler cannot prove the sign of an
+// operand (it then forms a 64-bit product of three instructions; fx_split hides
+// the sign of l).  mad.wide.s32 written as inline PTX is no help: half of its
+// additions become separate instructions (158 against 109 per five dot
+// products of five terms).
+__device__ __forceinline__ long long fx_madw(int a, int b, long long c) { return (long long)a * b + c; }
 
 __device__ __forceinline__ unsigned fx_hi(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
 
 // Block maximum of every lane's five m[v] into slot[v] (zero before; a
 // barrier must follow).
-__device__ __forceinline__ void fx_flush_max(const unsigned* m, unsigned* slot) {
+template <class I>
+__device__ __forceinline__ void fx_flush_max(const I* m, I* slot) {
   const int l32 = threadIdx.x & 31;
-  unsigned x = 0u;
+  I x = 0;
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
-    const unsigned r = __reduce_max_sync(0xffffffffu, m[v]);
+    const I r = __reduce_max_sync(0xffffffffu, m[v]);
     x = l32 == v ? r : x;
   }
   if (l32 < 5) atomicMax(slot + l32, x);
@@ -509,7 +518,7 @@ __device__ __forceinline__ void fx_to_nodal(const Ctx& c, const TypeTab& T, cons
     FxD d[n];
     const int eb = fx_load_aligned<n>(Y + v * nQ + jk, n2, e1 + v * n2 + k, n, d) + Tab::gA;
     double* o = bufA + v * nQ + jk;
-#pragma unroll
+#pragma unroll kUnroll
     for (int i = 0; i < n; ++i) o[i * n2] = fx_to(fx_dot<n>(d, [&](int p) { return Tab::A(p, i); }), eb);
     if (TR) {
       double x[n];
@@ -574,7 +583,7 @@ __device__ __forceinline__ void fx_modal_tail(const Ctx& c, const TypeTab& T, co
                    (ub ? 0 : __ldg(ip + T.col_s + col));
     if (uc) {
       double* o = r + v * nM + col * n;
-#pragma unroll
+#pragma unroll kUnroll
       for (int t = 0; t < n; ++t) o[t] = fx_to(fx_dot<n>(d, [&](int k) { return Tab::A(t, k); }), em + Tab::gA);
     } else {
       const int2* C = c.fpool + T.C + __ldg(ip + T.col_coff + col);
@@ -714,24 +723,14 @@ __device__ __forceinline__ void fx_lift_to_modal(const Ctx& c, const TypeTab& T,
 }
 
 // out = sum over the directions l in `dirs` of D_l^T G_l (collocation
-// derivative, G_l at G + 5 l nQ): out [5][nQ] (shared or global).  tmp
-// [5][nQ] scratch.  slot: set whose words hold the largest high word per
-// variable when `scanned`, else cleared and filled here.
-template <int n>
-__device__ __forceinline__ void fx_dsum_body(const double* G, unsigned dirs, double* tmp, double* out, unsigned* slot,
-                                             bool scanned) {
+// derivative): load(l, v, q) gives G_l at point q, read once; em(v) the exponent
+// all of them share, |G| < 2^(em + 1 - 1023).  out [5][nQ] (shared or global);
+// tmp [5][nQ] scratch.  A barrier stands between the writes of what load and em
+// read and this call.
+template <int n, class Load, class Em>
+__device__ __forceinline__ void fx_dsum(Load load, Em em, unsigned dirs, double* tmp, double* out) {
   constexpr int n2 = n * n, nQ = n2 * n;
   using Tab = FxTab<n>;
-  if (!scanned) {
-    fx_clear(slot, 5);
-    __syncthreads();
-    unsigned m[5] = {0u, 0u, 0u, 0u, 0u};
-#pragma unroll 1
-    for (int l = 0; l < 3; ++l)
-      if ((dirs >> l) & 1u) fx_scan(G + 5 * l * nQ, nQ, nQ, m);
-    fx_flush_max(m, slot);
-  }
-  __syncthreads();
   long long* A = reinterpret_cast<long long*>(tmp);
   bool first = true;
 #pragma unroll 1
@@ -742,23 +741,29 @@ __device__ __forceinline__ void fx_dsum_body(const double* G, unsigned dirs, dou
       const int v = t0 / n2;
       int st, sd, fp;
       fx_line_of<n>(l, t0 - v * n2, st, sd, fp);
-      const int em = fx_em(slot[v]) + 2;     // room for the three sums
-      const double* s = G + (5 * l + v) * nQ + st;
+      const int e = em(v) + 2;     // room for the three sums
       FxD d[n];
 #pragma unroll
-      for (int m = 0; m < n; ++m) d[m] = fx_split(fx_from(s[m * sd], em), 0);
+      for (int m = 0; m < n; ++m) d[m] = fx_split(fx_from(load(l, v, st + m * sd), e), 0);
       const int o = v * nQ + st;
-#pragma unroll
+#pragma unroll kUnroll
       for (int i = 0; i < n; ++i) {
         long long R = fx_dot<n>(d, [&](int m) { return Tab::D(i, m); }, Tab::S(i));
         if (!first) R += A[o + i * sd];
-        if (last) out[o + i * sd] = fx_to(R, em + 1 + Tab::gD);
+        if (last) out[o + i * sd] = fx_to(R, e + 1 + Tab::gD);
         else A[o + i * sd] = R;
       }
     }
     first = false;
     __syncthreads();
   }
+}
+
+// Exponent of a product f x from its factors' high words (at most one bit above
+// the product's own); a factor that is infinite or NaN marks the block.
+__device__ __forceinline__ int fx_em_product(double f, unsigned hx) {
+  const int ef = (int)(fx_hi(f) >> 20), ex = (int)(hx >> 20);
+  return ef == 2047 || ex == 2047 ? kFxBad + 2047 : ef + ex - 1022;
 }
 
 // dst_l = D_l src (the transposed derivative tables), l = 0..2: dst [3][5][nQ]
@@ -831,7 +836,7 @@ __device__ __forceinline__ void fx_lift(const TypeTab& T, double* buf, const dou
       if (lf0 >= 0) d[0] = fx_split(fx_from(F[(lf0 * 5 + v) * n2 + fp], em, neg), 0);
       if (lf1 >= 0) d[1] = fx_split(fx_from(F[(lf1 * 5 + v) * n2 + fp], em, neg), 0);
       const int o = v * nQ + st;
-#pragma unroll
+#pragma unroll kUnroll
       for (int i = 0; i < n; ++i) {
         long long R = l == 2 ? fx_from(buf[o + i * sd], em + kFxGE) : A[o + i * sd];
         R += fx_dot<2>(d, [&](int e) { return Tab::E(e, i); });
@@ -841,6 +846,76 @@ __device__ __forceinline__ void fx_lift(const TypeTab& T, double* buf, const dou
     }
     __syncthreads();
   }
+}
+
+// out(mode, acc[5]) = Md r: Md [nM][nM] doubles in global memory, symmetric and
+// positive definite (its largest entry is on the diagonal), r [5][nM] doubles
+// in shared memory (destroyed).  Both become 54-bit integers (rounded) in two 27-bit
+// halves: the four products of a term and their sums over nM <= 196 terms fit
+// 64 bits, so nothing is dropped or shifted before the end.  A lane owns a
+// mode: one load and conversion of Md feeds five variables.  FP64 took 5
+// multiply-adds per entry, 94 clocks of the SM per warp; this is about 45
+// instructions, and what bounds it is the latency of Md's loads (two curved
+// 12^3 steps at N = 4: 4.13 -> 4.06 ms; an L2 prefetch of Md at the start of the
+// phase made it 4.14, unrolling by 8 4.20).
+template <class Out>
+__device__ __forceinline__ void fx_dense(const double* Md, double* r, int nM, Out out) {
+  unsigned* sx = fx_slots();   // five words for r, one for Md
+  fx_clear(sx, 6);
+  __syncthreads();
+  unsigned m[5] = {0u, 0u, 0u, 0u, 0u}, md = 0u;
+  fx_scan(r, nM, nM, m);
+  for (int a = threadIdx.x; a < nM; a += blockDim.x) md = max(md, fx_hi(Md[(size_t)a * (nM + 1)]));
+  fx_flush_max(m, sx);
+  md = __reduce_max_sync(0xffffffffu, md);
+  if ((threadIdx.x & 31) == 0 && md) atomicMax(sx + 5, md);
+  __syncthreads();
+  constexpr int kLow = (1 << 27) - 1;
+  auto halves = [](long long D) {   // 55 bits -> 54, rounded
+    D = (D + 1) >> 1;
+    return make_int2((int)(D >> 27), (int)D & kLow);
+  };
+  int2* ri = reinterpret_cast<int2*>(r);
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    const int em = fx_em(sx[v]) + 6;
+    for (int a = threadIdx.x; a < nM; a += blockDim.x) ri[v * nM + a] = halves(fx_from(r[v * nM + a], em));
+  }
+  __syncthreads();
+  const int emd = fx_em(sx[5]) + 6;
+  for (int a = threadIdx.x; a < nM; a += blockDim.x) {
+    long long hh[5], mid[5], ll[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) hh[v] = mid[v] = ll[v] = 0;
+#pragma unroll 4
+    for (int j = 0; j < nM; ++j) {
+      int2 k = halves(fx_from(Md[(size_t)j * nM + a], emd));
+      asm("" : "+r"(k.y));   // see fx_madw
+#pragma unroll
+      for (int v = 0; v < 5; ++v) {
+        int2 d = ri[v * nM + j];
+        asm("" : "+r"(d.y));
+        hh[v] = fx_madw(d.x, k.x, hh[v]);
+        mid[v] = fx_madw(d.x, k.y, mid[v]);
+        mid[v] = fx_madw(d.y, k.x, mid[v]);
+        ll[v] = fx_madw(d.y, k.y, ll[v]);
+      }
+    }
+    double acc[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      // hh 2^54 + mid 2^27 + ll, |sum| < 2^116, as (hi, lo) = 2^27 hi + lo, then the top 64 bits
+      const long long t = mid[v] + (ll[v] >> 27);
+      const long long hi = hh[v] + (t >> 27);                    // units of 2^54
+      const unsigned lo = (unsigned)t & (unsigned)kLow;          // next 27 bits
+      const int ks = fx_shift(fx_mag(hi)), k = min(ks, 27);
+      const long long R = (hi << k) | (long long)(lo >> (27 - k));
+      // hi 2^54 units: value = hi 2^(54 - (1083 - em_r) - (1083 - em_d)); fx_to takes R 2^(eb - 1084)
+      acc[v] = fx_to(R, (fx_em(sx[v]) + 7) + (emd + 1) - 1028 - k);
+    }
+    out(a, acc);
+  }
+  __syncthreads();
 }
 
 }  // namespace
