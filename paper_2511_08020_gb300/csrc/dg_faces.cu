@@ -138,13 +138,14 @@ __global__ void face_ns_kernel(Ctx c) {
     }
     const bool cg = CURVED && R.cgeo >= 0;   // curved owner: per-point normal and w S
     const double wS = cg ? c.fgeo[R.cgeo + 3 * n2 + p] : c.dpool[c.tabs[R.owner_tab].fw + R.owner_lf * n2 + p] * R.S;
-    double Fs[5];
+    double Fs[5];   // w S times the value
     if (KIND == 0) {
       double WL[5], WR[5];
       primitive(UL, gm1, WL);
       primitive(UR, gm1, WR);
+      const double h = 0.5 * wS;
 #pragma unroll
-      for (int v = 0; v < 5; ++v) Fs[v] = 0.5 * (WL[v] + WR[v]);
+      for (int v = 0; v < 5; ++v) Fs[v] = h * (WL[v] + WR[v]);
     } else {
       double nrm[3] = {R.nrm[0], R.nrm[1], R.nrm[2]};
       if (cg) {
@@ -152,26 +153,51 @@ __global__ void face_ns_kernel(Ctx c) {
         nrm[1] = c.fgeo[R.cgeo + n2 + p];
         nrm[2] = c.fgeo[R.cgeo + 2 * n2 + p];
       }
-      if (CURVED && c.fmot && cg) {
-        // moving mesh: the LF flux in the frame of the normal mesh speed
-        const double* xf = c.fmot + 3 * (int64_t)R.cgeo + 9 * n2 + p;
-        const double sn = nrm[0] * xf[0] + nrm[1] * xf[n2] + nrm[2] * xf[2 * n2];
-        flux_lf_moving_scaled(UL, UR, nrm, 1.0, sn, gamma, Fs);
-      } else if (c.flux == 0) {
-        flux_lf(UL, UR, nrm, gamma, Fs);
+      // everything with the scaled normal s = (w S / 2) n: the inviscid flux as
+      // in flux_lf_scaled, the viscous one as the sum of both sides' F_v.s
+      const double h = 0.5 * wS;
+      const double s[3] = {h * nrm[0], h * nrm[1], h * nrm[2]};
+      double rL, pL, rR, pR;
+      if (c.flux == 0) {
+        LfSide L, Q;
+        if (CURVED && c.fmot && cg) {
+          // moving mesh: the LF flux in the frame of the normal mesh speed
+          const double* xf = c.fmot + 3 * (int64_t)R.cgeo + 9 * n2 + p;
+          const double sig = s[0] * xf[0] + s[1] * xf[n2] + s[2] * xf[2 * n2];
+          lf_side<true>(UL, s, h, sig, gm1, gamma, L);
+          lf_side<true>(UR, s, h, sig, gm1, gamma, Q);
+          lf_combine_moving(UL, UR, s, sig, L, Q, Fs);
+        } else {
+          lf_side<false>(UL, s, h, 0.0, gm1, gamma, L);
+          lf_side<false>(UR, s, h, 0.0, gm1, gamma, Q);
+          lf_combine(UL, UR, s, L, Q, Fs);
+        }
+        rL = L.r;
+        pL = L.p;
+        rR = Q.r;
+        pR = Q.p;
       } else {
         flux_roe(UL, UR, nrm, gamma, Fs);
+#pragma unroll
+        for (int v = 0; v < 5; ++v) Fs[v] *= wS;
+        double W[5];
+        primitive(UL, gm1, W);
+        rL = rcp(UL[0]);
+        pL = W[4];
+        primitive(UR, gm1, W);
+        rR = rcp(UR[0]);
+        pR = W[4];
       }
       const double* V0 = c.Vt + 3 * R.toff;
       const double* V1 = V0 + 15 * n2;
-      double g[15], W[5], Fv[3][5];
+      double g[15], u[3], q[4];
 #pragma unroll
       for (int t = 0; t < 15; ++t) g[t] = V0[t * n2 + p];
-      primitive(UL, gm1, W);
-      viscous_flux(W, g, c.mu, c.kappa, Fv);
-      double Fvn[5];
 #pragma unroll
-      for (int v = 0; v < 5; ++v) Fvn[v] = nrm[0] * Fv[0][v] + nrm[1] * Fv[1][v] + nrm[2] * Fv[2][v];
+      for (int d = 0; d < 3; ++d) u[d] = UL[1 + d] * rL;
+      viscous_flux_normal(rL, u, pL, g, s, c.mu, c.kappa, q);
+#pragma unroll
+      for (int v = 0; v < 4; ++v) Fs[1 + v] -= q[v];
       if (R.map >= 0) {
         int j = c.perms[(size_t)R.map + p];
 #pragma unroll
@@ -185,13 +211,11 @@ __global__ void face_ns_kernel(Ctx c) {
           g[t] = acc;
         }
       }
-      primitive(UR, gm1, W);
-      viscous_flux(W, g, c.mu, c.kappa, Fv);
 #pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        Fvn[v] += nrm[0] * Fv[0][v] + nrm[1] * Fv[1][v] + nrm[2] * Fv[2][v];
-        Fs[v] -= 0.5 * Fvn[v];
-      }
+      for (int d = 0; d < 3; ++d) u[d] = UR[1 + d] * rR;
+      viscous_flux_normal(rR, u, pR, g, s, c.mu, c.kappa, q);
+#pragma unroll
+      for (int v = 0; v < 4; ++v) Fs[1 + v] -= q[v];
     }
     if (R.map >= 0) {
       // permutation map: direct writes (this thread alone read the inputs at
@@ -201,12 +225,12 @@ __global__ void face_ns_kernel(Ctx c) {
       const double nb = KIND == 0 ? 1.0 : -1.0;
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        O0[v * n2 + p] = wS * Fs[v];
-        O0[(5 + v) * n2 + j] = nb * wS * Fs[v];
+        O0[v * n2 + p] = Fs[v];
+        O0[(5 + v) * n2 + j] = nb * Fs[v];
       }
     } else {
 #pragma unroll
-      for (int v = 0; v < 5; ++v) sF[(fl * 5 + v) * n2 + p] = wS * Fs[v];
+      for (int v = 0; v < 5; ++v) sF[(fl * 5 + v) * n2 + p] = Fs[v];
     }
   }
   __syncthreads();

@@ -71,85 +71,75 @@ __device__ __forceinline__ void normal_state(const double* U, const double* n, d
 }
 
 // Lax-Friedrichs: F* = (F- + F+)/2 - lambda (U+ - U-)/2,
-// lambda = max(|u-.n| + c-, |u+.n| + c+).
-__device__ __forceinline__ void flux_lf(const double* UL, const double* UR, const double* n, double gamma, double* Fs) {
-  NState L, R;
-  normal_state(UL, n, gamma, L);
-  normal_state(UR, n, gamma, R);
-  double cL = sqrt_hw(gamma * L.p * L.rinv), cR = sqrt_hw(gamma * R.p * R.rinv);
-  double lam = fmax(fabs(L.un) + cL, fabs(R.un) + cR);
+// lambda = max(|u-.n| + c-, |u+.n| + c+), multiplied by the face weight
+// wS = w S of the point and arranged for few FP64 instructions: with the scaled
+// normal s = (wS/2) n and us = m.s/rho per side,
+//   wS F*_rho = m-.s + m+.s + lam (rho- - rho+),
+//   wS F*_m   = m- us- + m+ us+ + (p- + p+) s + lam (m- - m+),
+//   wS F*_E   = (E- + p-) us- + (E+ + p+) us+ + lam (E- - E+),
+//   lam       = max(|us-| + (wS/2) c-, |us+| + (wS/2) c+),
+// one reciprocal and one square root per side.  fmax passes over the NaN of a
+// side whose pressure is negative, so the other side's speed is taken there.
+// The face kernel is bound by FP64 issue: about 75 instructions per point, 105
+// with IEEE division, root and separate side fluxes (16^3 mixed N = 4: 151 us,
+// 140 with the reciprocals alone, 130 in this form; the Navier-Stokes flux phase
+// at 12^3 164 -> 128 us).
+struct LfSide {
+  double r, p, ms, us, lam;
+};
+
+// sig: the face's normal mesh speed times wS/2 (moving meshes), else zero
+template <bool MOVING>
+__device__ __forceinline__ void lf_side(const double* U, const double* s, double h, double sig, double gm1,
+                                        double gamma, LfSide& o) {
+  o.r = rcp(U[0]);
+  o.ms = fma(U[1], s[0], fma(U[2], s[1], U[3] * s[2]));
+  o.us = o.ms * o.r;
+  const double m2 = fma(U[1], U[1], fma(U[2], U[2], U[3] * U[3]));
+  o.p = gm1 * fma(-0.5 * o.r, m2, U[4]);
+  o.lam = fma(h, sqrt_hw(gamma * o.p * o.r), fabs(MOVING ? o.us - sig : o.us));
+}
+
+__device__ __forceinline__ void lf_combine(const double* UL, const double* UR, const double* s, const LfSide& L,
+                                           const LfSide& R, double* Fs) {
+  const double lam = fmax(L.lam, R.lam), P = L.p + R.p;
+  Fs[0] = fma(lam, UL[0] - UR[0], L.ms + R.ms);
 #pragma unroll
-  for (int v = 0; v < 5; ++v) Fs[v] = 0.5 * (L.F[v] + R.F[v]) - 0.5 * lam * (UR[v] - UL[v]);
+  for (int d = 0; d < 3; ++d)
+    Fs[1 + d] = fma(lam, UL[1 + d] - UR[1 + d], fma(UL[1 + d], L.us, fma(UR[1 + d], R.us, P * s[d])));
+  Fs[4] = fma(lam, UL[4] - UR[4], fma(UL[4] + L.p, L.us, (UR[4] + R.p) * R.us));
 }
 
-// The Lax-Friedrichs flux above, already multiplied by the face weight
-// wS = w S of the point, arranged for few FP64 instructions: with the scaled
-// normal s = (wS/2) n,
-//   wS F* = F_s(U-) + F_s(U+) + lam_s (U- - U+),
-//   F_s(U) = (m.s, m (m.s)/rho + p s, (E + p)(m.s)/rho),
-//   lam_s = max(|m-.s|/rho- + (wS/2) c-, |m+.s|/rho+ + (wS/2) c+),
-// so rho F_0 = m.n needs no multiply, one reciprocal and one square root per
-// side serve the flux and the wave speed, and the 1/2 and wS scales fold into
-// the normal.
-__device__ __forceinline__ void lf_side(const double* U, const double* s, double h, double gm1, double gamma,
-                                        double* F, double& lam) {
-  const double r = rcp(U[0]);
-  const double ms = fma(U[1], s[0], fma(U[2], s[1], U[3] * s[2]));
-  const double us = ms * r;
-  const double m2 = fma(U[1], U[1], fma(U[2], U[2], U[3] * U[3]));
-  const double p = gm1 * fma(-0.5 * r, m2, U[4]);
-  F[0] = ms;
-  F[1] = fma(U[1], us, p * s[0]);
-  F[2] = fma(U[2], us, p * s[1]);
-  F[3] = fma(U[3], us, p * s[2]);
-  F[4] = (U[4] + p) * us;
-  lam = fma(h, sqrt_hw(gamma * p * r), fabs(us));
-}
-
-__device__ __forceinline__ void moving_lf_side(const double* U, const double* s, double h, double sig, double gm1,
-                                               double gamma, double* F, double& lam) {
-  const double r = rcp(U[0]);
-  const double ms = fma(U[1], s[0], fma(U[2], s[1], U[3] * s[2]));
-  const double us = ms * r;
-  const double m2 = fma(U[1], U[1], fma(U[2], U[2], U[3] * U[3]));
-  const double p = gm1 * fma(-0.5 * r, m2, U[4]);
-  const double ur = us - sig;
-  F[0] = fma(-sig, U[0], ms);
-  F[1] = fma(U[1], ur, p * s[0]);
-  F[2] = fma(U[2], ur, p * s[1]);
-  F[3] = fma(U[3], ur, p * s[2]);
-  F[4] = fma(U[4], ur, p * us);
-  lam = fma(h, sqrt_hw(gamma * p * r), fabs(ur));
+// The same in a frame moving with normal speed sn = xdot.n at the point: the
+// side fluxes lose sig U, sig = (wS/2) sn.
+__device__ __forceinline__ void lf_combine_moving(const double* UL, const double* UR, const double* s, double sig,
+                                                  const LfSide& L, const LfSide& R, double* Fs) {
+  const double lam = fmax(L.lam, R.lam), P = L.p + R.p, wL = L.us - sig, wR = R.us - sig;
+  Fs[0] = fma(lam, UL[0] - UR[0], fma(-sig, UL[0], L.ms) + fma(-sig, UR[0], R.ms));
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+    Fs[1 + d] = fma(lam, UL[1 + d] - UR[1 + d], fma(UL[1 + d], wL, fma(UR[1 + d], wR, P * s[d])));
+  Fs[4] = fma(lam, UL[4] - UR[4], fma(UL[4], wL, fma(UR[4], wR, fma(L.p, L.us, R.p * R.us))));
 }
 
 __device__ __forceinline__ void flux_lf_scaled(const double* UL, const double* UR, const double* n, double wS,
                                                double gamma, double* Fs) {
-  const double h = 0.5 * wS;
+  const double h = 0.5 * wS, gm1 = gamma - 1.0;
   const double s[3] = {h * n[0], h * n[1], h * n[2]};
-  const double gm1 = gamma - 1.0;
-  double FL[5], FR[5], lamL, lamR;
-  lf_side(UL, s, h, gm1, gamma, FL, lamL);
-  lf_side(UR, s, h, gm1, gamma, FR, lamR);
-  const double lam = fmax(lamL, lamR);
-#pragma unroll
-  for (int v = 0; v < 5; ++v) Fs[v] = fma(lam, UL[v] - UR[v], FL[v] + FR[v]);
+  LfSide L, R;
+  lf_side<false>(UL, s, h, 0.0, gm1, gamma, L);
+  lf_side<false>(UR, s, h, 0.0, gm1, gamma, R);
+  lf_combine(UL, UR, s, L, R, Fs);
 }
 
-// The same flux in a frame moving with normal speed sn = xdot.n at the point
-// (moving meshes): F_s(U) - sig U with sig = (wS/2) sn, and the wave speed
-// from the relative normal velocity, lam_s = max(|m.s/rho - sig| + (wS/2) c).
 __device__ __forceinline__ void flux_lf_moving_scaled(const double* UL, const double* UR, const double* n, double wS,
                                                       double sn, double gamma, double* Fs) {
-  const double h = 0.5 * wS;
+  const double h = 0.5 * wS, gm1 = gamma - 1.0, sig = h * sn;
   const double s[3] = {h * n[0], h * n[1], h * n[2]};
-  const double sig = h * sn;
-  const double gm1 = gamma - 1.0;
-  double FL[5], FR[5], lamL, lamR;
-  moving_lf_side(UL, s, h, sig, gm1, gamma, FL, lamL);
-  moving_lf_side(UR, s, h, sig, gm1, gamma, FR, lamR);
-  const double lam = fmax(lamL, lamR);
-#pragma unroll
-  for (int v = 0; v < 5; ++v) Fs[v] = fma(lam, UL[v] - UR[v], FL[v] + FR[v]);
+  LfSide L, R;
+  lf_side<true>(UL, s, h, sig, gm1, gamma, L);
+  lf_side<true>(UR, s, h, sig, gm1, gamma, R);
+  lf_combine_moving(UL, UR, s, sig, L, R, Fs);
 }
 
 // Roe: F* = (F- + F+)/2 - sum_k |lambda_k| alpha_k r_k / 2 with
@@ -357,6 +347,28 @@ __device__ __forceinline__ void viscous_flux(const double* W, const double* g, d
   }
 }
 
+// Viscous flux through a face, F_v.s for a (scaled) normal s, from 1/rho, the
+// velocity, p and the gradient: q[0..2] momentum, q[3] energy.  The traction is
+// contracted with s before the stress is formed (41 FP64 instructions; the
+// three fluxes and their contraction took about 75).
+__device__ __forceinline__ void viscous_flux_normal(double r, const double* u, double p, const double* g,
+                                                    const double* s, double mu, double kappa, double* q) {
+  const double lam = (2.0 / 3.0) * mu * (g[1] + g[5 + 2] + g[10 + 3]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    double a = s[0] * g[1 + i];
+    a = fma(s[1], g[5 + 1 + i], a);
+    a = fma(s[2], g[10 + 1 + i], a);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) a = fma(s[d], g[i * 5 + 1 + d], a);
+    q[i] = fma(mu, a, -lam * s[i]);
+  }
+  const double gp = fma(s[0], g[4], fma(s[1], g[9], s[2] * g[14]));
+  const double gr = fma(s[0], g[0], fma(s[1], g[5], s[2] * g[10]));
+  const double dT = fma(-p * r, gr, gp) * r;
+  q[3] = fma(kappa, dT, fma(u[0], q[0], fma(u[1], q[1], u[2] * q[2])));
+}
+
 // Reverse mode of viscous_flux: Fb[d][v] cotangent of F_v[d][v]; adds the
 // cotangents of W (5) to Wb and of the gradient (15) to gb.
 __device__ __forceinline__ void viscous_flux_vjp(const double* W, const double* g, double mu, double kappa,
@@ -475,7 +487,7 @@ __device__ __forceinline__ void flux_lf_vjp(const double* UL, const double* UR, 
   const double aLb = aL >= aR ? lamb : 0.0, aRb = aL >= aR ? 0.0 : lamb;
   // c = sqrt(gamma p / rho): dc = gamma dp / (2 c rho) - c drho / (2 rho)
   double ubL[3] = {0, 0, 0}, ubR[3] = {0, 0, 0};
-  const double pbL = aLb * gamma * L.rinv / (2.0 * cL), pbR = aRb * gamma * R.rinv / (2.0 * cR);
+  const double pbL = 0.5 * aLb * gamma * L.rinv * rcp(cL), pbR = 0.5 * aRb * gamma * R.rinv * rcp(cR);
   UbL[0] -= aLb * 0.5 * cL * L.rinv;
   UbR[0] -= aRb * 0.5 * cR * R.rinv;
   normal_state_vjp(UL, n, gamma, L, Fb, sgn0(L.un) * aLb, pbL, 0.0, ubL, UbL);
@@ -588,7 +600,7 @@ __device__ __forceinline__ void flux_roe_vjp(const double* UL, const double* UR,
 #pragma unroll
   for (int d = 0; d < 3; ++d) ub[d] += unb * n[d];
   // c = sqrt(c2), c2 = (gamma-1)(H - q2/2), q2 = |u|^2
-  c2b += cb / (2.0 * c);
+  c2b += 0.5 * cb * rcp(c);
   Hb += gm1 * c2b;
   q2b -= 0.5 * gm1 * c2b;
 #pragma unroll
@@ -610,8 +622,8 @@ __device__ __forceinline__ void flux_roe_vjp(const double* UL, const double* UR,
   }
   sLb -= denb * den * den;
   sRb -= denb * den * den;
-  UbL[0] += sLb / (2.0 * sL) - drhob;
-  UbR[0] += sRb / (2.0 * sR) + drhob;
+  UbL[0] += 0.5 * sLb * rcp(sL) - drhob;
+  UbR[0] += 0.5 * sRb * rcp(sR) + drhob;
   normal_state_vjp(UL, n, gamma, L, FbL, 0.0, -dpb, HLb, ubL, UbL);
   normal_state_vjp(UR, n, gamma, R, FbR, 0.0, dpb, HRb, ubR, UbR);
 }
