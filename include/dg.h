@@ -541,8 +541,8 @@ dg_status dg_set_scheduler(dg_mesh* mesh, int scheduler);
 
 /* Tile shape of the element kernels: the number of warps (1..4) that work
  * together on one element (one element per thread block), for every (type,
- * N) table at once.  The default is 2 for N <= 2, 3 for N = 3 and 4
- * above; dg_autotune
+ * N) table at once.  The default is 2 for N <= 2, 3 for N = 3 and 4 above, and
+ * 4 for every N on meshes of at most four elements per SM; dg_autotune
  * picks the fastest.  Rebuilds the chunk tables; results are bitwise
  * identical for every choice. */
 dg_status dg_set_element_warps(dg_mesh* mesh, int warps);

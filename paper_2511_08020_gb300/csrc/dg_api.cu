@@ -1174,8 +1174,14 @@ namespace {
 // Warps per element for n points per direction: the lines of a pass (5 n^2
 // lanes' worth of work) per block.  Measured on mixed meshes (step, two warps
 // / chosen): n = 4 1848 / 1805 us, n = 5 7058 / 6406 us, n = 6 viscous
-// 4394 / 3508 us; n <= 3 is within 2% from two to four warps.
-int default_warps(int n) { return n <= 3 ? 2 : (n == 4 ? 3 : 4); }
+// 4394 / 3508 us; n <= 3 is within 2% from two to four warps.  A mesh of a few
+// elements per SM waits for each element's chain of phases, which more lanes
+// shorten: four warps there (residual of 4^3 cubes of four types, N = 2: 78 us
+// with two, 73 with four).
+int default_warps(int n, int64_t n_elems, int num_sms) {
+  if (n_elems <= 4 * (int64_t)num_sms) return 4;
+  return n <= 3 ? 2 : (n == 4 ? 3 : 4);
+}
 
 dg_status create_device_mesh(dg_mesh* m, const dg_mesh_desc* desc, cudaStream_t stream, dg_mesh** out) {
   m->flux = desc->flux;
@@ -1186,7 +1192,7 @@ dg_status create_device_mesh(dg_mesh* m, const dg_mesh_desc* desc, cudaStream_t 
   cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, m->device);
   const dgh::HostMesh& h = m->h;
   m->nQmax = h.n * h.n * h.n;
-  m->wpb = default_warps(h.n);  // warps cooperating on one element
+  m->wpb = default_warps(h.n, h.n_elems, m->num_sms);  // warps cooperating on one element
   auto fail_cuda = [&](cudaError_t e, const char* what) {
     m->release();
     delete m;
@@ -1237,7 +1243,7 @@ dg_status create_device_mesh(dg_mesh* m, const dg_mesh_desc* desc, cudaStream_t 
     const std::vector<double> w0 = m->static_weights();
     for (int t = 0; t < dgk::kMaxTabs; ++t) {
       m->weight[t] = w0[t];
-      m->tab_wpb[t] = t < (int)h.tables.tabs.size() ? default_warps(h.tables.tabs[t].n) : m->wpb;
+      m->tab_wpb[t] = t < (int)h.tables.tabs.size() ? default_warps(h.tables.tabs[t].n, h.n_elems, m->num_sms) : m->wpb;
     }
   }
   if ((e = m->build_groups()) != cudaSuccess) return fail_cuda(e, "chunk table");
