@@ -34,13 +34,20 @@ enum Family { kStage = 0, kNs = 1, kMisc = 2 };
 // more than a few spilled registers: 16^3 mixed N = 4, two steps, 5.83 / 5.63 /
 // 5.52 ms with 6 / 7 / 8 blocks; N = 5 and 6 are limited by shared memory.
 constexpr int kStageBlocks = kn <= 5 ? 8 : 5, kNsBlocks = kn <= 5 ? 6 : (kn == 6 ? 4 : 2);
+// The split-form volume term holds the states of a line in registers and shared
+// memory limits it anyway.  One step of hexahedra, 4 / 5 / 8 blocks: n = 2
+// (16^3) 1339 / 1174 / 1163 us, n = 3 (12^3) 1046 / 1040 / 1163 and 928 with 6,
+// n = 4 (10^3) 1016 / 1111 / 1252, n = 5 (9^3) 2088 / 1563 / 1569: four are the
+// faster there while the last wave is full (10^3 mixed 1396 / 1668 / 1678), five
+// never lose to the FP64 kernel (1635 and 2001).
+constexpr int kSplitBlocks = kn <= 3 ? 6 : (kn == 4 ? 4 : 5);
 
 // ------------------------------------------------------------------ element phases
 //
-// Every pass gives one lane one output point and carries the 5 conservative
-// variables in registers: one coefficient load feeds 5 independent FMA chains
-// (instruction-level parallelism for the FP64 pipe) and the index arithmetic
-// is done once per output.  Buffers are [var][point] with a var stride of nQ.
+// The contractions run on the integer pipe (dg_fixed.cuh); what stays on FP64
+// is the pointwise physics and the conversions.  Buffers are [var][point] with
+// a var stride of nQ.  The few FP64 dot products left carry the 5 variables in
+// registers, so one coefficient load feeds 5 independent FMA chains.
 
 #define DG_FMA5(cf, src, stride, acc)            \
   do {                                           \
@@ -1370,7 +1377,7 @@ __device__ __forceinline__ StageArgs resolve_args(const StageArgs& a) {
 // One element per block (chunk_start null: the listed slots), or a persistent
 // launch whose blocks pop chunks of the list from the queue.
 template <int FAM, bool ANY, bool SPLIT>
-__global__ void __launch_bounds__(128, FAM == kStage ? kStageBlocks : (FAM == kNs ? kNsBlocks : 1)) elem_kernel(const __grid_constant__ Ctx c, int mode,
+__global__ void __launch_bounds__(128, FAM == kStage ? (SPLIT ? kSplitBlocks : kStageBlocks) : (FAM == kNs ? kNsBlocks : 1)) elem_kernel(const __grid_constant__ Ctx c, int mode,
                                                    const __grid_constant__ StageArgs io0,
                                                    const __grid_constant__ Sched sc) {
   extern __shared__ double smem[];

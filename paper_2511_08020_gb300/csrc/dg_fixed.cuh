@@ -19,8 +19,8 @@
 // every line with its own exponent, taken from its results (the OR of their
 // magnitudes): the collapsed bases grow towards the degenerate edge where the
 // weighted data shrink, so one exponent per element would cost the bits that
-// the next pass needs there (measured: 5 to 10 times the FP64 passes' error at
-// N = 6, with an exponent per line two thirds of it).  Sums of several
+// the next pass needs there (measured, residual at N = 6: FP64 passes 3.5e-12,
+// one exponent 2.5e-11, an exponent per line 2.8e-12).  Sums of several
 // directions (the derivative sum, the lift) share one exponent per variable.
 //
 // A lane owns one line of n points of one variable: it reads the n values
