@@ -220,17 +220,16 @@ FACE_POINT_FLOPS_NS = {"lift": 36, "lf": 101 + 2 * (13 + 66 + 30) + 10, "roe": 2
 # (backward + LSERK + forward) of this workload, from the committed ncu
 # capture of the element kernel on the 16^3 N = 4 mesh; set to None whenever
 # the element kernel changes until it is captured again.
-NCU_TRAFFIC_FUSED_LAUNCH = (154.316032 + 144.723456) * 1e6
+NCU_TRAFFIC_FUSED_LAUNCH = None
 # the same capture's executed FP64 rate: (2 DFMA + DMUL + DADD thread
 # instructions per cycle, all SMs) x the SM clock of the launch, and the FP64
 # pipe's busy fraction (the same rule: None once the kernel changes)
-NCU_FP64_FUSED_LAUNCH = {"executed_tflops": (2 * 215.843480 + 31.503288 + 1.640137) * 2.073804e9 / 1e12,
-                         "fp64_pipe_busy": 0.92798396}
+NCU_FP64_FUSED_LAUNCH = None
 # dram__bytes_read.sum + dram__bytes_write.sum of one stage solve of the
 # moving leg (its launches for hexahedra, prisms and pyramids), from the
 # committed ncu capture of the mass kernel on the 16^3 N = 4 mesh in motion;
 # None whenever the mass kernel changes until it is captured again.
-NCU_TRAFFIC_MASS_SOLVE = (10.084608 + (210.038528 + 16.756480) + (233.019648 + 95.310336)) * 1e6
+NCU_TRAFFIC_MASS_SOLVE = None
 
 
 def fp64_probes():
@@ -940,7 +939,8 @@ def run_ours_legs(args, dg, torch, ws, rank, local, box, dev, stream, barrier, m
                      "achieved": elem_tflops, "peak": peak_derived, "unit": "TFLOP/s",
                      "frac": elem_tflops / peak_derived,
                      "peak_kind": f"derived: {props.multi_processor_count} SMs x 2 DFMA/clk x 2 flop x "
-                                  f"{sm_max_ghz:.3f} GHz (max SM clock of the run)",
+                                  f"{sm_max_ghz:.3f} GHz (max SM clock of the run); the kernel's contractions "
+                                  "run as integer multiply-adds, so its FP64-equivalent rate may exceed it",
                      "dfma_loop_measured": dfma, "frac_of_dfma_loop": elem_tflops / dfma,
                      "traffic": NCU_TRAFFIC_FUSED_LAUNCH,
                      "ncu_fp64": NCU_FP64_FUSED_LAUNCH,
