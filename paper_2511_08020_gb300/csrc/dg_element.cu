@@ -1879,12 +1879,13 @@ cudaError_t mass(const Ctx& c, const int64_t* list, int64_t n_slots, const doubl
   };
   // rows per lane in the warp solves and the panel (nM <= 32 ROWS): two up to
   // N = 3 and for pyramids of N = 4, three for prisms of N = 4 and pyramids of
-  // N = 5, four for prisms of N = 5 (moving meshes end there)
+  // N = 5, four for prisms of N = 5 (moving prisms and pyramids end there).
+  // Hexahedra (max_nM = 0, pointwise, every N) run in the degree's smallest.
   cudaError_t e = cudaErrorInvalidValue;
-  if constexpr (kn <= 5) {
-    if (max_nM <= 64) e = launch(moving_mass_kernel<2, kMassBlocks2>);
-  } else if constexpr (kn == 6) {
+  if constexpr (kn == 6) {
     if (max_nM <= 64) e = launch(moving_mass_kernel<3, kMassBlocks>);
+  } else {
+    if (max_nM <= (kn <= 5 ? 64 : 0)) e = launch(moving_mass_kernel<2, kMassBlocks2>);
   }
   if constexpr (kn == 5 || kn == 6)
     if (max_nM > 64 && max_nM <= 96) e = launch(moving_mass_kernel<3, kMassBlocks>);
