@@ -60,13 +60,18 @@ def build_probe(force: bool = False) -> str:
     return PROBE_LIB
 
 
+def dependencies() -> list:
+    """Every file libdg.so is made from (sources, headers, this file with its flags and build list)."""
+    srcs = [os.path.join(CSRC, s) for s in (*SOURCES, ELEMENT_SRC)]
+    srcs += [os.path.join(CSRC, h) for h in sorted(os.listdir(CSRC)) if h.endswith((".h", ".cuh"))]
+    return srcs + [os.path.join(ROOT, "include", "dg.h"), os.path.abspath(__file__)]
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(LIBDIR, exist_ok=True)
-    srcs = [os.path.join(CSRC, s) for s in SOURCES] + [os.path.join(CSRC, h) for h in os.listdir(CSRC) if h.endswith((".h", ".cuh"))]
-    srcs.append(os.path.join(ROOT, "include", "dg.h"))
     if not force and os.path.exists(LIB):
         lib_t = os.path.getmtime(LIB)
-        if all(os.path.getmtime(s) <= lib_t for s in srcs):
+        if all(os.path.getmtime(s) <= lib_t for s in dependencies()):
             return LIB
     jobs = [(ELEMENT_SRC, f"dg_element_{n}_{p}", (f"-DDG_N={n}", f"-DDG_PART={p}")) for n, p in ELEMENT_BUILDS]
     jobs += [(s, os.path.splitext(s)[0], ()) for s in SOURCES]
