@@ -438,7 +438,6 @@ __device__ __forceinline__ void element_forward_t(const Ctx& c, const TypeTab& T
                                                   int lane) {
   constexpr int n = kn, nQ = knQ, n2 = kn2;
   const double* dp = c.dpool;
-  fx_clear(fx_slots() + 10, 5);
   if (T.type == HEX) {
     modal_to_nodal(c, T, bufG, bufA, bufG, lane);
     write_traces(c, T, s, bufA, c.T);
@@ -471,11 +470,7 @@ __device__ __forceinline__ void element_forward_t(const Ctx& c, const TypeTab& T
   // moving mesh: the mesh velocity at the volume points
   const double* xd = (curved && c.mpool) ? c.mpool + c.slot_moff[s] + 31 * nQ : nullptr;
   const double gm1 = c.gamma - 1.0;
-  unsigned mg[5] = {0u, 0u, 0u, 0u, 0u};   // largest high words of G per variable
-  auto put = [&](double* G, int v, double x) {
-    G[v * nQ] = x;
-    mg[v] = max(mg[v], fx_hi(x));
-  };
+  auto put = [&](double* G, int v, double x) { G[v * nQ] = x; };
   for (int q = lane; q < nQ; q += blockDim.x) {
     double U[5];
 #pragma unroll
@@ -520,12 +515,11 @@ __device__ __forceinline__ void element_forward_t(const Ctx& c, const TypeTab& T
       put(G, 4, Vl * Ep);
     }
   }
-  fx_flush_max(mg, fx_slots() + 10);
   // H = sum_l D_l^T G_l (collocation derivative along each collapsed direction)
   // (the last direction's sums run in place of its own G)
   __syncthreads();
-  fx_dsum<kn>([&](int l, int v, int q) { return bufG[(5 * l + v) * nQ + q]; },
-              [&](int v) { return fx_em(fx_slots()[10 + v]); }, 7u, bufG + 10 * nQ, c.H + c.slot_hoff[s]);
+  fx_dsum<kn>([&](int l, int v, int q) { return bufG[(5 * l + v) * nQ + q]; }, 7u, bufG + 10 * nQ,
+              c.H + c.slot_hoff[s]);
 }
 
 template <bool ANY, bool SPLIT>
@@ -677,7 +671,6 @@ __device__ __forceinline__ void element_ns_volume_t(const Ctx& c, const TypeTab&
     for (int v = 0; v < 5; ++v) bufA[v * nQ + q] = W[v];
   }
   const unsigned nz = kMetricMask[T.type];
-  int* es = reinterpret_cast<int*>(fx_slots()) + 10;
 #pragma unroll 1
   for (int k = 0; k < 3; ++k) {
     // affine: P_k; a curved element takes one full set of directional passes
@@ -686,22 +679,9 @@ __device__ __forceinline__ void element_ns_volume_t(const Ctx& c, const TypeTab&
     auto metric = [&](int l, int q) {
       return CURVED ? cblk[(l * 3 + k) * nQ + q] : __ldg(dp + T.wA + q * 9 + l * 3 + k);
     };
-    if (lane < 5) es[lane] = -4096;
     __syncthreads();
-    {
-      int m[5] = {-4096, -4096, -4096, -4096, -4096};
-      for (int q = lane; q < nQ; q += blockDim.x)
-        for (int l = 0; l < 3; ++l) {
-          if (!((dirs >> l) & 1u)) continue;
-          const double f = metric(l, q);
-#pragma unroll
-          for (int v = 0; v < 5; ++v) m[v] = max(m[v], fx_em_product(f, fx_hi(bufA[v * nQ + q])));
-        }
-      fx_flush_max(m, es);
-    }
-    __syncthreads();
-    fx_dsum<kn>([&](int l, int v, int q) { return metric(l, q) * bufA[v * nQ + q]; }, [&](int v) { return es[v]; }, dirs,
-                bufG + 5 * nQ, CURVED ? bufDW + k * 5 * nQ : bufG);
+    fx_dsum<kn>([&](int l, int v, int q) { return metric(l, q) * bufA[v * nQ + q]; }, dirs, bufG + 5 * nQ,
+                CURVED ? bufDW + k * 5 * nQ : bufG);
     if (!CURVED) {
       for (int w = lane; w < 5 * nQ; w += blockDim.x) {
         const double p = bufG[w];
@@ -771,11 +751,7 @@ __device__ __forceinline__ void element_ns_volume_t(const Ctx& c, const TypeTab&
   // (in place of the point's gradient)
   fx_clear(fx_slots() + 10, 5);
   __syncthreads();
-  unsigned mg[5] = {0u, 0u, 0u, 0u, 0u};   // largest high words of G per variable
-  auto put = [&](double* G, int v, double x) {
-    G[v * nQ] = x;
-    mg[v] = max(mg[v], fx_hi(x));
-  };
+  auto put = [&](double* G, int v, double x) { G[v * nQ] = x; };
   for (int q = lane; q < nQ; q += blockDim.x) {
     double U[5], W[5], gr[15];
 #pragma unroll
@@ -823,10 +799,8 @@ __device__ __forceinline__ void element_ns_volume_t(const Ctx& c, const TypeTab&
       put(G, 4, Vl * Ep - (M[l][0] * Fv[0][4] + M[l][1] * Fv[1][4] + M[l][2] * Fv[2][4]));
     }
   }
-  fx_flush_max(mg, fx_slots() + 10);
   __syncthreads();
-  fx_dsum<kn>([&](int l, int v, int q) { return bufDW[(5 * l + v) * nQ + q]; },
-              [&](int v) { return fx_em(fx_slots()[10 + v]); }, 7u, bufG, c.H + c.slot_hoff[s]);
+  fx_dsum<kn>([&](int l, int v, int q) { return bufDW[(5 * l + v) * nQ + q]; }, 7u, bufG, c.H + c.slot_hoff[s]);
 }
 
 template <bool ANY>

@@ -20,8 +20,9 @@
 // magnitudes): the collapsed bases grow towards the degenerate edge where the
 // weighted data shrink, so one exponent per element would cost the bits that
 // the next pass needs there (measured, residual at N = 6: FP64 passes 3.5e-12,
-// one exponent 2.5e-11, an exponent per line 2.8e-12).  Sums of several
-// directions (the derivative sum, the lift) share one exponent per variable.
+// one exponent 2.5e-11, an exponent per line 2.8e-12).  In the
+// derivative sum every line keeps its own too and the directions meet on the
+// largest at a point; the lift shares one per variable.
 //
 // A lane owns one line of n points of one variable: it reads the n values
 // once and forms all n results, so the coefficients are the same for every
@@ -723,47 +724,64 @@ __device__ __forceinline__ void fx_lift_to_modal(const Ctx& c, const TypeTab& T,
 }
 
 // out = sum over the directions l in `dirs` of D_l^T G_l (collocation
-// derivative): load(l, v, q) gives G_l at point q, read once; em(v) the exponent
-// all of them share, |G| < 2^(em + 1 - 1023).  out [5][nQ] (shared or global);
-// tmp [5][nQ] scratch.  A barrier stands between the writes of what load and em
-// read and this call.
-template <int n, class Load, class Em>
-__device__ __forceinline__ void fx_dsum(Load load, Em em, unsigned dirs, double* tmp, double* out) {
+// derivative): load(l, v, q) gives G_l at point q, read once.  out [5][nQ]
+// (shared or global); tmp [5][nQ] scratch, which may be G_2 itself.  Every line
+// keeps the exponent of its own values: a hexahedron's results are its nodal
+// rates, and those of a line of small values are not to depend on a large value
+// elsewhere in the element.  The directions' sums meet at a point on the largest
+// of the exponents of the lines through it.
+template <int n, class Load>
+__device__ __forceinline__ void fx_dsum(Load load, unsigned dirs, double* tmp, double* out) {
   constexpr int n2 = n * n, nQ = n2 * n;
   using Tab = FxTab<n>;
   long long* A = reinterpret_cast<long long*>(tmp);
+  int* es = fx_exps<n>();   // the lines' exponents: direction 2, direction 1
   bool first = true;
 #pragma unroll 1
   for (int l = 2; l >= 0; --l) {
     if (!((dirs >> l) & 1u)) continue;
     const bool last = (dirs & ((1u << l) - 1u)) == 0u;
+    // exponent of the sum so far at point m of a line: max(ea[m sa], eb[m sb]) + room
+    const bool two = l == 0 && (dirs & 6u) == 6u;
+    const bool by1 = l == 0 && !(dirs & 4u);
     for (int t0 = threadIdx.x; t0 < 5 * n2; t0 += blockDim.x) {
-      const int v = t0 / n2;
+      const int v = t0 / n2, id = t0 - v * n2, x1 = id / n, x2 = id - x1 * n;
       int st, sd, fp;
-      fx_line_of<n>(l, t0 - v * n2, st, sd, fp);
-      const int e = em(v) + 2;     // room for the three sums
-      FxD d[n];
+      fx_line_of<n>(l, id, st, sd, fp);
+      double x[n];
 #pragma unroll
-      for (int m = 0; m < n; ++m) d[m] = fx_split(fx_from(load(l, v, st + m * sd), e), 0);
+      for (int m = 0; m < n; ++m) x[m] = load(l, v, st + m * sd);
+      FxD d[n];
+      const int eb = fx_line<n>(x, d) + 1 + Tab::gD;
       const int o = v * nQ + st;
+      if (first) {
 #pragma unroll kUnroll
-      for (int i = 0; i < n; ++i) {
-        long long R = fx_dot<n>(d, [&](int m) { return Tab::D(i, m); }, Tab::S(i));
-        if (!first) R += A[o + i * sd];
-        if (last) out[o + i * sd] = fx_to(R, e + 1 + Tab::gD);
-        else A[o + i * sd] = R;
+        for (int i = 0; i < n; ++i) {
+          const long long R = fx_dot<n>(d, [&](int m) { return Tab::D(i, m); }, Tab::S(i));
+          if (last) out[o + i * sd] = fx_to(R, eb);
+          else A[o + i * sd] = R;
+        }
+      } else {
+        // the lines through a point of this one: direction 2 (x_0, x_1), direction 1 (x_0, x_2)
+        const int* e2 = es + v * n2 + (l == 1 ? x1 * n : x1);
+        const int* e1 = es + (5 + v) * n2 + x2;
+        const int* p = by1 ? e1 : e2;
+        const int* q = two ? e1 : p;
+        const int se = l == 1 ? 1 : n;
+#pragma unroll kUnroll
+        for (int i = 0; i < n; ++i) {
+          const long long R = fx_dot<n>(d, [&](int m) { return Tab::D(i, m); }, Tab::S(i));
+          const int ep = max(p[i * se], q[i * se]) + (two ? 1 : 0), e = max(ep, eb) + 1;
+          const long long r = (A[o + i * sd] >> min(e - ep, 63)) + (R >> min(e - eb, 63));
+          if (last) out[o + i * sd] = fx_to(r, e);
+          else A[o + i * sd] = r;
+        }
       }
+      if (!last) es[(l == 2 ? 0 : 5 * n2) + v * n2 + id] = eb;
     }
     first = false;
     __syncthreads();
   }
-}
-
-// Exponent of a product f x from its factors' high words (at most one bit above
-// the product's own); a factor that is infinite or NaN marks the block.
-__device__ __forceinline__ int fx_em_product(double f, unsigned hx) {
-  const int ef = (int)(fx_hi(f) >> 20), ex = (int)(hx >> 20);
-  return ef == 2047 || ex == 2047 ? kFxBad + 2047 : ef + ex - 1022;
 }
 
 // dst_l = D_l src (the transposed derivative tables), l = 0..2: dst [3][5][nQ]
