@@ -531,38 +531,30 @@ __device__ __forceinline__ void element_forward(const Ctx& c, const TypeTab& T, 
 
 // Backward phase, first half: bufA = H +- sum_faces E_f^T F_f with the
 // face values F_f read from `faces` (the lifted fluxes, subtracted with neg
-// 0x80000000; the adjoint's trace cotangents, added with neg 0).  They are staged into bufG with
-// coalesced loads first.
+// 0x80000000; the adjoint's trace cotangents, added with neg 0).  H and F are
+// staged into bufG with coalesced loads first (H is read in place for n = 2,
+// where bufG holds the face values only).
 template <bool ANY>
 __device__ __forceinline__ void element_lift(const Ctx& c, const TypeTab& T, int64_t s, double* bufA, double* bufG,
                                             int lane, const double* faces, unsigned neg, const double* pscale) {
-  constexpr int n = kn, nQ = knQ, n2 = kn2;
+  constexpr int nQ = knQ, n2 = kn2;
+  constexpr bool room = 30 * n2 + 5 * nQ <= 15 * nQ;
   const int nf = T.nfaces;
   const int64_t* ft = c.slot_ftoff + s * 6;
-  fx_clear(fx_slots() + 5, 5);
-  unsigned m[5] = {0u, 0u, 0u, 0u, 0u};
   const double* H = c.H + c.slot_hoff[s];
+  double* sH = bufG + 30 * n2;
+  for (int w = lane; w < 5 * nQ && room; w += blockDim.x) sH[w] = H[w];
 #pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    for (int q = lane; q < nQ; q += blockDim.x) {
-      const double x = H[v * nQ + q];
-      bufA[v * nQ + q] = x;
-      m[v] = max(m[v], fx_hi(x));
-    }
+  for (int v = 0; v < 5; ++v)
     for (int w = lane; w < nf * n2; w += blockDim.x) {
       const int lf = w / n2, o = v * n2 + w - lf * n2;
-      const double x = faces[ft[lf] + o];
-      bufG[lf * 5 * n2 + o] = x;
-      m[v] = max(m[v], fx_hi(x));
+      bufG[lf * 5 * n2 + o] = faces[ft[lf] + o];
     }
-  }
   __syncthreads();
-  fx_lift<kn>(T, bufA, bufG, neg, m);
-  if (ANY && pscale) {
+  fx_lift<kn>(T, [&](int o) { return room ? sH[o] : H[o]; }, bufG, neg, bufA, [&](int o, double x) {
     // curved hexahedron: M^{-1} V^T = V^T diag(1/J) (V square, V^T W V = I)
-    for (int w = lane; w < 5 * nQ; w += blockDim.x) bufA[w] *= pscale[w % nQ];
-    __syncthreads();
-  }
+    bufA[o] = ANY && pscale ? x * pscale[o % nQ] : x;
+  });
 }
 
 // Backward phase of the element: r = V^T (H +- sum_f E_f^T F_f) through `ep`.
@@ -584,32 +576,26 @@ __device__ __forceinline__ bool element_backward(const Ctx& c, const TypeTab& T,
   return ANY && ep.Md ? finish_modal<true>(c, T, r, lane, ep) : finish_modal<false>(c, T, r, lane, ep);
 }
 
-// BR1 lifting face term: bufA += sum_f coef_f E_f^T L_f with coef_f =
-// sign n_d(f), n(f) the element's outward unit normal of local face f and
-// L_f the face values at its own points (staged through bufS).
-template <bool CURVED>
-__device__ __forceinline__ void lift_scaled_t(const Ctx& c, const TypeTab& T, int64_t s, double* bufA, double* bufS,
-                                           int lane, const double* faces, int d, double sign) {
-  constexpr int n = kn, n2 = kn2;
+// BR1 lifting face term of a hexahedron: out(o, dW(o) - sum_f n_d(f) E_f^T L_f),
+// n(f) the element's outward unit normal of local face f and L_f the face
+// values at its own points (staged through bufS; bufA scratch).
+template <bool CURVED, class Out>
+__device__ __forceinline__ void lift_scaled_t(const Ctx& c, const TypeTab& T, int64_t s, const double* dW, double* bufA,
+                                           double* bufS, int lane, const double* faces, int d, Out out) {
+  constexpr int n2 = kn2;
   const int nf = T.nfaces;
   const int64_t* ft = c.slot_ftoff + s * 6;
   // the normal multiplies the staged face values (curved: point by point,
   // c.snrm holds each side's own normals)
-  fx_clear(fx_slots() + 5, 5);
-  unsigned m[5] = {0u, 0u, 0u, 0u, 0u};
 #pragma unroll
-  for (int v = 0; v < 5; ++v) {
+  for (int v = 0; v < 5; ++v)
     for (int w = lane; w < nf * n2; w += blockDim.x) {
       const int lf = w / n2, p = w - lf * n2, o = v * n2 + p;
       const double nd = CURVED ? c.snrm[3 * (ft[lf] / 5) + d * n2 + p] : c.fnrm[(s * 6 + lf) * 3 + d];
-      const double x = sign * nd * faces[ft[lf] + o];
-      bufS[lf * 5 * n2 + o] = x;
-      m[v] = max(m[v], fx_hi(x));
+      bufS[lf * 5 * n2 + o] = nd * faces[ft[lf] + o];
     }
-  }
-  fx_scan(bufA, knQ, knQ, m);
   __syncthreads();
-  fx_lift<kn>(T, bufA, bufS, 0u, m);
+  fx_lift<kn>(T, [&](int o) { return dW[o]; }, bufS, 0x80000000u, bufA, out);
 }
 
 // Navier-Stokes volume phase of the element at slot s (after the lifting face
@@ -699,19 +685,13 @@ __device__ __forceinline__ void element_ns_volume_t(const Ctx& c, const TypeTab&
   for (int d = 0; d < 3; ++d) {
     double* dW = bufDW + d * 5 * nQ;
     if (T.type == HEX) {
-      for (int w = lane; w < 5 * nQ; w += blockDim.x) bufA[w] = dW[w];
-      __syncthreads();
-      lift_scaled_t<CURVED>(c, T, s, bufA, bufG, lane, c.L, d, -1.0);
       // V is square for the hexahedron, so V M^{-1} V^T = (W J)^{-1}: the
       // projection onto the modal space is the identity at the nodes
       const double* wq = dp + T.W;
-      if (CURVED) {
-        const double* iJ = cblk + 10 * nQ;
-        for (int w = lane; w < 5 * nQ; w += blockDim.x) dW[w] = -iJ[w % nQ] * bufA[w] * rcp(wq[w % nQ]);
-      } else {
-        for (int w = lane; w < 5 * nQ; w += blockDim.x) dW[w] = -g.invJ * bufA[w] * rcp(wq[w % nQ]);
-      }
-      __syncthreads();
+      const double* iJ = CURVED ? cblk + 10 * nQ : nullptr;
+      lift_scaled_t<CURVED>(c, T, s, dW, bufA, bufG, lane, c.L, d, [&](int o, double x) {
+        dW[o] = -(CURVED ? iJ[o % nQ] : g.invJ) * x * rcp(wq[o % nQ]);
+      });
       write_traces(c, T, s, dW, c.Vt, 0u, 3, (int64_t)d * 5 * n2);
     } else {
       // r = V^T (Hd - sum_f n_d(f) E_f^T L_f), then the projection
@@ -1083,24 +1063,19 @@ __device__ __forceinline__ void element_vjp_c(const Ctx& c, const VjpArgs& va, i
 //   C (shared with Euler): Qbar = V^T (Ubar + sum_f E_f^T Tbar_f).
 
 // bufA += sum_f E_f^T faces_f, face values at (ft_mult ft[lf] + ft_add)
-// (staged through bufS).
-__device__ __forceinline__ void lift_add(const Ctx& c, const TypeTab& T, int64_t s, double* bufA, double* bufS, int lane,
-                                      const double* faces, int ft_mult, int64_t ft_add) {
+// (staged through bufS; bufX [5 nQ] scratch).
+__device__ __forceinline__ void lift_add(const Ctx& c, const TypeTab& T, int64_t s, double* bufA, double* bufS,
+                                      double* bufX, int lane, const double* faces, int ft_mult, int64_t ft_add) {
   const int nf = T.nfaces;
   const int64_t* ft = c.slot_ftoff + s * 6;
-  fx_clear(fx_slots() + 5, 5);
-  unsigned m[5] = {0u, 0u, 0u, 0u, 0u};
 #pragma unroll
   for (int v = 0; v < 5; ++v)
     for (int w = lane; w < nf * kn2; w += blockDim.x) {
       const int lf = w / kn2, o = v * kn2 + w - lf * kn2;
-      const double x = faces[ft_mult * ft[lf] + ft_add + o];
-      bufS[lf * 5 * kn2 + o] = x;
-      m[v] = max(m[v], fx_hi(x));
+      bufS[lf * 5 * kn2 + o] = faces[ft_mult * ft[lf] + ft_add + o];
     }
-  fx_scan(bufA, knQ, knQ, m);
   __syncthreads();
-  fx_lift<kn>(T, bufA, bufS, 0u, m);
+  fx_lift<kn>(T, [&](int o) { return bufA[o]; }, bufS, 0u, bufX, [&](int o, double x) { bufA[o] = x; });
 }
 
 // Phase A (Navier-Stokes).  smem: bufY [5 nQ] | bufG [15 nQ] | bufS [5 nQ].
@@ -1221,7 +1196,7 @@ __device__ __forceinline__ void element_vjp_b_ns_t(const Ctx& c, int64_t s, doub
   constexpr int n = kn, nQ = knQ, n2 = kn2;
   const int nf = T.nfaces;
   constexpr int nQm = knQ;
-  double* bufD = smem;                 // smem + 15 nQm .. 20 nQm is unused
+  double* bufD = smem;                 // smem + 15 nQm .. 20 nQm is scratch
   double* bufX = smem + 20 * nQm;
   double* bufW = smem + 25 * nQm;
   double* bufL = smem + 30 * nQm;
@@ -1233,7 +1208,7 @@ __device__ __forceinline__ void element_vjp_b_ns_t(const Ctx& c, int64_t s, doub
     for (int w = lane; w < 15 * nQ; w += blockDim.x) bufD[w] = DWs[w];
   }
   __syncthreads();
-  for (int d = 0; d < 3; ++d) lift_add(c, T, s, bufD + d * 5 * nQ, bufL, lane, c.Vtb, 3, (int64_t)d * 5 * n2);
+  for (int d = 0; d < 3; ++d) lift_add(c, T, s, bufD + d * 5 * nQ, bufL, smem + 15 * nQm, lane, c.Vtb, 3, (int64_t)d * 5 * n2);
   for (int w = lane; w < 5 * nQ; w += blockDim.x) bufW[w] = 0.0;
   for (int w = lane; w < nf * 5 * n2; w += blockDim.x) bufL[w] = 0.0;
   __syncthreads();

@@ -21,8 +21,9 @@
 // weighted data shrink, so one exponent per element would cost the bits that
 // the next pass needs there (measured, residual at N = 6: FP64 passes 3.5e-12,
 // one exponent 2.5e-11, an exponent per line 2.8e-12).  In the
-// derivative sum every line keeps its own too and the directions meet on the
-// largest at a point; the lift shares one per variable.
+// derivative sum and in the lift at a node every line keeps its own too, and what
+// meets at a point meets on the largest there; the lift that goes on into a
+// transform shares one per variable.
 //
 // A lane owns one line of n points of one variable: it reads the n values
 // once and forms all n results, so the coefficients are the same for every
@@ -828,39 +829,54 @@ __device__ __forceinline__ void fx_grad1(int l, const double* src, double* dst) 
   __syncthreads();
 }
 
-// buf += sum_f E_f^T (+-F_f): buf [5][nQ] doubles in place, F [nf][5][n^2]
-// doubles (both shared); neg 0x80000000 subtracts.  m: this lane's maxima of
-// the high words of buf and F (any partition of them over the lanes); the
-// words fx_slots() + 5 are clear, with a barrier since.
-template <int n>
-__device__ __forceinline__ void fx_lift(const TypeTab& T, double* buf, const double* F, unsigned neg,
-                                        const unsigned* m) {
+// out(o, h) with h = H(o) + sum_f E_f^T (+-F_f) at every node o = v nQ + q: F
+// [nf][5][n^2] doubles (shared); neg 0x80000000 subtracts; A [5][nQ] scratch.
+// The lane that puts out(o) reads H(o) just before, so out may write where H
+// reads, or to A.  The two face values at the ends of a line share an exponent,
+// and the sums meet H at each node on the largest of that node's own.
+template <int n, class LoadH, class Out>
+__device__ __forceinline__ void fx_lift(const TypeTab& T, LoadH H, const double* F, unsigned neg, double* scratch,
+                                        Out out) {
   constexpr int n2 = n * n, nQ = n2 * n;
   using Tab = FxTab<n>;
-  unsigned* sx = fx_slots() + 5;
-  fx_flush_max(m, sx);
-  __syncthreads();
-  long long* A = reinterpret_cast<long long*>(buf);
+  long long* A = reinterpret_cast<long long*>(scratch);
+  int* es = fx_exps<n>();   // the lines' exponents: direction 2, direction 1
 #pragma unroll 1
   for (int l = 2; l >= 0; --l) {
     const int lf0 = T.face_of[2 * l], lf1 = T.face_of[2 * l + 1];
     for (int t0 = threadIdx.x; t0 < 5 * n2; t0 += blockDim.x) {
-      const int v = t0 / n2;
+      const int v = t0 / n2, id = t0 - v * n2, x1 = id / n, x2 = id - x1 * n;
       int st, sd, fp;
-      fx_line_of<n>(l, t0 - v * n2, st, sd, fp);
-      const int em = fx_em(sx[v]);
+      fx_line_of<n>(l, id, st, sd, fp);
+      double f[2];
+      f[0] = lf0 >= 0 ? F[(lf0 * 5 + v) * n2 + fp] : 0.0;
+      f[1] = lf1 >= 0 ? F[(lf1 * 5 + v) * n2 + fp] : 0.0;
+      // 62 bits of each value: two end coefficients sum to less than 2, so a
+      // line's results stay below 2^60, and three of them with H below 2^63
       FxD d[2];
-      d[0] = d[1] = FxD{0, 0};
-      if (lf0 >= 0) d[0] = fx_split(fx_from(F[(lf0 * 5 + v) * n2 + fp], em, neg), 0);
-      if (lf1 >= 0) d[1] = fx_split(fx_from(F[(lf1 * 5 + v) * n2 + fp], em, neg), 0);
+      const int em = fx_em(max(fx_hi(f[0]), fx_hi(f[1]))), eb = em + kFxGE;
+      d[0] = fx_split(fx_from(f[0], em, neg), 1);
+      d[1] = fx_split(fx_from(f[1], em, neg), 1);
       const int o = v * nQ + st;
+      // the lines through a point of this one: direction 2 (x_0, x_1), direction 1 (x_0, x_2)
+      const int* e2 = es + v * n2 + (l == 1 ? x1 * n : x1);
+      const int* e1 = es + (5 + v) * n2 + x2;
 #pragma unroll kUnroll
       for (int i = 0; i < n; ++i) {
-        long long R = l == 2 ? fx_from(buf[o + i * sd], em + kFxGE) : A[o + i * sd];
-        R += fx_dot<2>(d, [&](int e) { return Tab::E(e, i); });
-        if (l == 0) buf[o + i * sd] = fx_to(R, em + 1 + kFxGE);
-        else A[o + i * sd] = R;
+        const long long R = fx_dot<2>(d, [&](int e) { return Tab::E(e, i); });
+        long long& a = A[o + i * sd];
+        if (l == 2) {
+          a = R;
+        } else if (l == 1) {
+          const int ep = e2[i], e = max(ep, eb);
+          a = (a >> min(e - ep, 63)) + (R >> min(e - eb, 63));
+        } else {
+          const double h = H(o + i * sd);
+          const int ep = max(e2[i * n], e1[i * n]), e = max(max(ep, eb), fx_em(fx_hi(h)) + 1);
+          out(o + i * sd, fx_to((a >> min(e - ep, 63)) + (R >> min(e - eb, 63)) + fx_from(h, e - 1), e));
+        }
       }
+      if (l > 0) es[(l == 2 ? 0 : 5 * n2) + v * n2 + id] = eb;
     }
     __syncthreads();
   }

@@ -64,6 +64,12 @@ template <int n> void dsum(const double* G, unsigned dirs, double* out) {
   double tmp[m];
   fx_dsum<n>([&](int l, int v, int q) { return g[(5 * l + v) * n * n * n + q]; }, dirs, (dirs & 4u) ? g + 2 * m : tmp, out);
 }
+template <int n> void lift(int type, const double* H, const double* F, int neg, double* out) {
+  constexpr int m = 5 * n * n * n;
+  Setup s(type, n - 1);
+  double A[m];
+  fx_lift<n>(s.T, [&](int o) { return H[o]; }, F, neg ? 0x80000000u : 0u, A, [&](int o, double x) { out[o] = x; });
+}
 template <int n> int nodal(int type, const double* Q, double* out, double* tr) {
   constexpr int n2 = n * n, m = 5 * n * n2;
   Setup s(type, n - 1);
@@ -87,6 +93,7 @@ template <int n> void grad(const double* U, double* out) { fx_grad<n>(U, out); }
 #define EACH(n, f) (n == 2 ? f<2> : n == 3 ? f<3> : n == 4 ? f<4> : n == 5 ? f<5> : n == 6 ? f<6> : f<7>)
 extern "C" {
 void t_dsum(int n, const double* G, unsigned dirs, double* out) { EACH(n, dsum)(G, dirs, out); }
+void t_lift(int n, int type, const double* H, const double* F, int neg, double* out) { EACH(n, lift)(type, H, F, neg, out); }
 int t_nodal(int n, int type, const double* Q, double* out, double* tr) { return EACH(n, nodal)(type, Q, out, tr); }
 int t_modal(int n, int type, const double* U, double* out) { return EACH(n, modal)(type, U, out); }
 void t_grad(int n, const double* U, double* out) { EACH(n, grad)(U, out); }

@@ -5,7 +5,7 @@ magnitudes."""
 import numpy as np
 import pytest
 
-from fixed_host import fx, nodes, ptr  # noqa: F401
+from fixed_host import fx, nodes, ptr, tables  # noqa: F401
 
 U = 2.0 ** -53
 DEGREES = range(2, 8)
@@ -36,3 +36,42 @@ def test_derivative_sum_keeps_line_scales(fx, n):  # noqa: F811
                 size += np.moveaxis((np.abs(g) * np.abs(D).astype(float)).sum(-2), -1, 1 + l)
         assert (np.abs(out - ref) <= (n + 3) * U * size).all()
         assert (out[4] == 0).all()
+
+
+def lifted(n, face, H, F, sign):
+    """h = H + sign sum_f E_f^T F_f and the sum of its terms' magnitudes."""
+    E = nodes(n)[2]
+    h, size = H.astype(LD), np.abs(H)
+    for l in range(3):
+        for end in range(2):
+            lf = face[2 * l + end]
+            if lf < 0:
+                continue
+            shape = [1, 1, 1, 1]
+            shape[1 + l] = n
+            # face point x1 + n x2 of the two other coordinates
+            term = sign * E[end].reshape(shape) * np.expand_dims(np.swapaxes(F[lf], 1, 2), 1 + l)
+            h, size = h + term, size + np.abs(term).astype(float)
+    return h, size
+
+
+def spread(rng, n, nf):
+    """Nodal values, and face values, of sizes from 1e-12 to 1: along a, and from node to node."""
+    H = rng.uniform(-1, 1, (5, n, n, n)) * 10.0 ** rng.uniform(-12, 0, (5, n, n, n))
+    F = rng.uniform(-1, 1, (nf, 5, n, n)) * 10.0 ** rng.uniform(-12, 0, (nf, 5, n, n))
+    return H, F
+
+
+@pytest.mark.parametrize("n", DEGREES)
+@pytest.mark.parametrize("etype", range(4))
+def test_lift_keeps_node_scales(fx, n, etype):  # noqa: F811
+    rng = np.random.default_rng(10 * n + etype)
+    face = tables(fx, n, etype)[1]
+    H, F = spread(rng, n, face.max() + 1)
+    for neg in (0, 1):
+        out = np.empty_like(H)
+        fx.t_lift(n, etype, ptr(H), ptr(F), neg, ptr(out))
+        h, size = lifted(n, face, H, F, -1 if neg else 1)
+        # besides the chain's nine roundings up to five units of 2^-57 of the largest value at the node, which
+        # counts there with a coefficient of min |E| at least
+        assert (np.abs(out - h) <= (9 + 5 / 16 / float(np.abs(nodes(n)[2]).min())) * U * size).all()
