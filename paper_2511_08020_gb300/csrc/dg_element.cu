@@ -571,7 +571,7 @@ __device__ __forceinline__ bool element_backward(const Ctx& c, const TypeTab& T,
   double* r = ANY && ep.Md ? ep.rbuf : bufA;
   const double* H = c.H + c.slot_hoff[s];
   const int64_t* ft = c.slot_ftoff + s * 6;
-  fx_lift_to_modal<kn>(c, T, [&](int o) { return H[o]; },
+  fx_lift_to_modal<kn, true>(c, T, [&](int o) { return H[o]; },
                        [&](int lf, int v, int p) { return faces[__ldg(ft + lf) + v * kn2 + p]; }, neg, bufA, bufG, r);
   return ANY && ep.Md ? finish_modal<true>(c, T, r, lane, ep) : finish_modal<false>(c, T, r, lane, ep);
 }
@@ -696,7 +696,7 @@ __device__ __forceinline__ void element_ns_volume_t(const Ctx& c, const TypeTab&
     } else {
       // r = V^T (Hd - sum_f n_d(f) E_f^T L_f), then the projection
       const int64_t* ft = c.slot_ftoff + s * 6;
-      fx_lift_to_modal<kn>(
+      fx_lift_to_modal<kn, false>(
           c, T, [&](int o) { return dW[o]; },
           [&](int lf, int v, int p) {
             const int64_t t = __ldg(ft + lf);

@@ -21,9 +21,11 @@
 // weighted data shrink, so one exponent per element would cost the bits that
 // the next pass needs there (measured, residual at N = 6: FP64 passes 3.5e-12,
 // one exponent 2.5e-11, an exponent per line 2.8e-12).  In the
-// derivative sum and in the lift at a node every line keeps its own too, and what
-// meets at a point meets on the largest there; the lift that goes on into a
-// transform shares one per variable.
+// derivative sum and the lift every line keeps its own too, and what meets at a
+// point (in the lift that goes on into a transform, on a line) meets on the
+// largest there: an element with a front in it holds lines of values 1e4 (1e12)
+// times below its largest, whose derivatives one exponent per variable left
+// 1e-12 (2e-4) of their size off at n = 5.
 //
 // A lane owns one line of n points of one variable: it reads the n values
 // once and forms all n results, so the coefficients are the same for every
@@ -317,10 +319,11 @@ __device__ __forceinline__ void fx_clear(unsigned* slot, int cnt) {
   for (int t = threadIdx.x; t < cnt; t += blockDim.x) slot[t] = 0u;
 }
 
-// Exponents of the lines between two passes
+// Exponents of the lines between two passes: two sets of [5][n^2] lines, the
+// second also as [4][5][n] lines of face values
 template <int n>
 __device__ __forceinline__ int* fx_exps() {
-  __shared__ int e[10 * n * n];
+  __shared__ int e[5 * n * n + (n < 4 ? 20 * n : 5 * n * n)];
   return e;
 }
 
@@ -627,69 +630,85 @@ __device__ __forceinline__ void fx_to_modal(const TypeTab& T, const Ctx& c, doub
 }
 
 // r = V^T (H +- sum_f E_f^T F_f) of a prism, pyramid or tetrahedron: H(o) the
-// nodal value at v nQ + q, F(f, v, p) the face values (read once each); neg
+// nodal value at v nQ + q, F(f, v, p) the face values (each read once); neg
 // 0x80000000 subtracts.  The sum stays in integers between the lift and the
 // transform: a lane owns the line (j, k), takes its n values of H, adds the b
 // and c face values with the two end coefficients of its j and k and the a
-// face values with the line's, and goes on with the a-pass.  bufA, bufG
-// [5][nQ] and F's [nf][5][n^2] at bufG (scratch); r [5][nM] may be bufA or lie
-// behind bufG's first 5 nQ.
-template <int n, class LoadH, class LoadF>
+// face values with the line's, and goes on with the a-pass.  A line of face
+// values along i keeps its own exponent, and the lane works on the largest of
+// what meets on its line.  bufA [5][nQ], bufG [30 n^2] scratch (STAGE: H lies in
+// global memory and is staged in bufA with the face values); r [5][nM] may be
+// bufA or lie behind bufG's first 5 nQ.
+template <int n, bool STAGE, class LoadH, class LoadF>
 __device__ __forceinline__ void fx_lift_to_modal(const Ctx& c, const TypeTab& T, LoadH H, LoadF F, unsigned neg,
                                                  double* bufA, double* bufG, double* r) {
   constexpr int n2 = n * n, nQ = n2 * n;
   using Tab = FxTab<n>;
-  unsigned* sx = fx_slots();
   int* e0 = fx_exps<n>();
-  const int nf = T.nfaces, nt = blockDim.x;
+  int* ef = e0 + 5 * n2;                 // [end][5][n] exponents of the b and c face lines
+  const int nt = blockDim.x;
   long long* Y = reinterpret_cast<long long*>(bufA);
-  long long* FI = reinterpret_cast<long long*>(bufG);
-  fx_clear(sx, 5);
-  unsigned m[5] = {0u, 0u, 0u, 0u, 0u};
-#pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    for (int q = threadIdx.x; q < nQ; q += nt) m[v] = max(m[v], fx_hi(H(v * nQ + q)));
-    for (int w = threadIdx.x; w < nf * n2; w += nt) {
-      const int lf = w / n2, p = w - lf * n2;
-      const double x = F(lf, v, p);
-      bufG[(lf * 5 + v) * n2 + p] = x;
-      m[v] = max(m[v], fx_hi(x));
-    }
-  }
-  __syncthreads();
-  fx_flush_max(m, sx);
-  __syncthreads();
-  // the face values as integers, in place (each lane the values it stored)
-  for (int v = 0; v < 5; ++v) {
-    const int em = fx_em(sx[v]);
-    for (int w = threadIdx.x; w < nf * n2; w += nt) {
-      const int lf = w / n2, o = lf * 5 * n2 + v * n2 + w - lf * n2;
-      FI[o] = fx_from(bufG[o], em, neg);
-    }
-  }
-  __syncthreads();
+  long long* FI = reinterpret_cast<long long*>(bufG);   // [end][5][n^2], ends -b, +b, -c, +c
+  double* FA = bufG + 20 * n2;                          // [2][5][n^2], ends -a, +a
   const int fa0 = __ldg(&T.face_of[0]), fa1 = __ldg(&T.face_of[1]);
+  for (int t0 = threadIdx.x; t0 < 5 * n2; t0 += nt) {
+    const int v = t0 / n2, jk = t0 - v * n2, j = jk / n, k = jk - j * n;
+    if (STAGE) {
+#pragma unroll
+      for (int i = 0; i < n; ++i) bufA[v * nQ + jk + i * n2] = H(v * nQ + jk + i * n2);
+    }
+    FA[t0] = F(fa0, v, j + n * k);
+    FA[5 * n2 + t0] = F(fa1, v, j + n * k);
+  }
+  for (int t0 = threadIdx.x; t0 < 20 * n; t0 += nt) {
+    const int e = t0 / (5 * n), w = t0 - e * 5 * n, v = w / n, y = w - v * n;
+    const int lf = __ldg(&T.face_of[2 + e]);
+    if (lf < 0) continue;
+    double x[n];
+    unsigned m = 0u;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      x[i] = F(lf, v, n * y + i);
+      m = max(m, fx_hi(x[i]));
+    }
+    const int em = fx_em(m);
+#pragma unroll
+    for (int i = 0; i < n; ++i) FI[(e * 5 + v) * n2 + n * y + i] = fx_from(x[i], em, neg);
+    ef[t0] = em;
+  }
+  __syncthreads();
   const int2* E = c.fpool + T.ext;
   for (int t0 = threadIdx.x; t0 < 5 * n2; t0 += nt) {
     const int v = t0 / n2, jk = t0 - v * n2, j = jk / n, k = jk - j * n;
-    const int em = fx_em(sx[v]);
+    const double a0 = FA[t0], a1 = FA[5 * n2 + t0];
+    double h[n];
+    unsigned m = max(fx_hi(a0), fx_hi(a1));
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      h[i] = STAGE ? bufA[v * nQ + jk + i * n2] : H(v * nQ + jk + i * n2);
+      m = max(m, fx_hi(h[i]));
+    }
+    int em = fx_em(m);
+#pragma unroll 1
+    for (int e = 0; e < 4; ++e)
+      if (__ldg(&T.face_of[2 + e]) >= 0) em = max(em, ef[(e * 5 + v) * n + (e < 2 ? k : j)]);
     long long mid[n], hh[n], half = kFxHalf;
 #pragma unroll
     for (int i = 0; i < n; ++i) {
-      hh[i] = fx_from(H(v * nQ + jk + i * n2), em + kFxGE);
+      hh[i] = fx_from(h[i], em + kFxGE);
       mid[i] = 0;
     }
     // b faces (line value at (i, k), coefficient of j), then c faces ((i, j), of k)
 #pragma unroll 1
     for (int e = 0; e < 4; ++e) {
-      const int lf = __ldg(&T.face_of[2 + e]);
-      if (lf < 0) continue;
+      if (__ldg(&T.face_of[2 + e]) < 0) continue;
       const int2 co = __ldg(E + (e & 1) * n + (e < 2 ? j : k));
-      const long long* f = FI + (lf * 5 + v) * n2 + n * (e < 2 ? k : j);
+      const int fl = e * 5 + v, y = e < 2 ? k : j, sh = min(em - ef[fl * n + y], 63);
+      const long long* f = FI + fl * n2 + n * y;
       half += co.y >> 1;   // the mean of the dl cl products (S above)
 #pragma unroll
       for (int i = 0; i < n; ++i) {
-        const FxD d = fx_split(f[i], 0);
+        const FxD d = fx_split(f[i] >> sh, 0);
         mid[i] = fx_madw(d.h, co.y, mid[i]);
         mid[i] = fx_madw(d.l, co.x, mid[i]);
         hh[i] = fx_madw(d.h, co.x, hh[i]);
@@ -697,16 +716,16 @@ __device__ __forceinline__ void fx_lift_to_modal(const Ctx& c, const TypeTab& T,
     }
     unsigned mg = 0u;
     {
-      const FxD a0 = fx_split(FI[(fa0 * 5 + v) * n2 + j + n * k], 0), a1 = fx_split(FI[(fa1 * 5 + v) * n2 + j + n * k], 0);
+      const FxD d0 = fx_split(fx_from(a0, em, neg), 0), d1 = fx_split(fx_from(a1, em, neg), 0);
 #pragma unroll
       for (int i = 0; i < n; ++i) {
         const int2 c0 = Tab::E(0, i), c1 = Tab::E(1, i);
-        mid[i] = fx_madw(a0.h, c0.y, mid[i]);
-        mid[i] = fx_madw(a0.l, c0.x, mid[i]);
-        mid[i] = fx_madw(a1.h, c1.y, mid[i]);
-        mid[i] = fx_madw(a1.l, c1.x, mid[i]);
-        hh[i] = fx_madw(a0.h, c0.x, hh[i]);
-        hh[i] = fx_madw(a1.h, c1.x, hh[i]);
+        mid[i] = fx_madw(d0.h, c0.y, mid[i]);
+        mid[i] = fx_madw(d0.l, c0.x, mid[i]);
+        mid[i] = fx_madw(d1.h, c1.y, mid[i]);
+        mid[i] = fx_madw(d1.l, c1.x, mid[i]);
+        hh[i] = fx_madw(d0.h, c0.x, hh[i]);
+        hh[i] = fx_madw(d1.h, c1.x, hh[i]);
         hh[i] += (mid[i] + half + ((c0.y + c1.y) >> 1)) >> 31;
         mg |= fx_mag(hh[i]);
       }

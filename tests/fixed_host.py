@@ -70,6 +70,17 @@ template <int n> void lift(int type, const double* H, const double* F, int neg, 
   double A[m];
   fx_lift<n>(s.T, [&](int o) { return H[o]; }, F, neg ? 0x80000000u : 0u, A, [&](int o, double x) { out[o] = x; });
 }
+template <int n> int lift_modal(int type, const double* H, const double* F, int neg, int stage, double* out) {
+  constexpr int m = 5 * n * n * n, g = 15 * n * n * n > 30 * n * n ? 15 * n * n * n : 30 * n * n;
+  Setup s(type, n - 1);
+  double A[m], G[g];
+  auto fH = [&](int o) { return H[o]; };
+  auto fF = [&](int lf, int v, int p) { return F[(lf * 5 + v) * n * n + p]; };
+  if (stage) fx_lift_to_modal<n, true>(s.c, s.T, fH, fF, neg ? 0x80000000u : 0u, A, G, A);
+  else fx_lift_to_modal<n, false>(s.c, s.T, fH, fF, neg ? 0x80000000u : 0u, A, G, G + m);
+  memcpy(out, stage ? A : G + m, 5 * s.T.nM * sizeof(double));
+  return s.T.nM;
+}
 template <int n> int nodal(int type, const double* Q, double* out, double* tr) {
   constexpr int n2 = n * n, m = 5 * n * n2;
   Setup s(type, n - 1);
@@ -94,6 +105,9 @@ template <int n> void grad(const double* U, double* out) { fx_grad<n>(U, out); }
 extern "C" {
 void t_dsum(int n, const double* G, unsigned dirs, double* out) { EACH(n, dsum)(G, dirs, out); }
 void t_lift(int n, int type, const double* H, const double* F, int neg, double* out) { EACH(n, lift)(type, H, F, neg, out); }
+int t_lift_modal(int n, int type, const double* H, const double* F, int neg, int stage, double* out) {
+  return EACH(n, lift_modal)(type, H, F, neg, stage, out);
+}
 int t_nodal(int n, int type, const double* Q, double* out, double* tr) { return EACH(n, nodal)(type, Q, out, tr); }
 int t_modal(int n, int type, const double* U, double* out) { return EACH(n, modal)(type, U, out); }
 void t_grad(int n, const double* U, double* out) { EACH(n, grad)(U, out); }

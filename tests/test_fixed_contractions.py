@@ -75,3 +75,23 @@ def test_lift_keeps_node_scales(fx, n, etype):  # noqa: F811
         # besides the chain's nine roundings up to five units of 2^-57 of the largest value at the node, which
         # counts there with a coefficient of min |E| at least
         assert (np.abs(out - h) <= (9 + 5 / 16 / float(np.abs(nodes(n)[2]).min())) * U * size).all()
+
+
+@pytest.mark.parametrize("n", DEGREES)
+@pytest.mark.parametrize("etype", range(4))
+def test_lift_to_modal_keeps_line_scales(fx, n, etype):  # noqa: F811
+    rng = np.random.default_rng(10 * n + etype)
+    V, face = tables(fx, n, etype)
+    nf, nM = face.max() + 1, V.shape[1]
+    H = rng.uniform(-1, 1, (5, n, n, n)) * 10.0 ** rng.uniform(-12, 0, (5, 1, n, n))
+    F = rng.uniform(-1, 1, (nf, 5, n, n)) * 10.0 ** rng.uniform(-12, 0, (nf, 5, n, 1))
+    for neg in (0, 1):
+        h, size = lifted(n, face, H, F, -1 if neg else 1)
+        ref = h.reshape(5, -1) @ V.astype(LD)
+        # what meets on a line along a shares an exponent
+        line = np.broadcast_to(size.max(axis=1, keepdims=True), size.shape)
+        bound = (3 * n + 9) * U * (line.reshape(5, -1) @ np.abs(V))
+        for stage in (0, 1):
+            out = np.empty((5, nM))
+            assert fx.t_lift_modal(n, etype, ptr(H), ptr(F), neg, stage, ptr(out)) == nM
+            assert (np.abs(out - ref) <= bound).all()
