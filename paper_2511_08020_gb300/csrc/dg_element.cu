@@ -153,10 +153,7 @@ __device__ __forceinline__ bool finish_modal(const Ctx& c, const TypeTab& T, dou
     bad |= epilogue_mode(ep, nM, mode, acc);
   }
   if (DENSE) {
-    // dense inverse mass matrix of a curved element (Algorithm 1 with a
-    // pointwise J): lanes run over output modes, so the column reads of the
-    // symmetric Md are coalesced and every load feeds 5 sums
-    fx_dense(ep.Md, r, nM, [&](int mode, double* acc) {
+    dense_product(ep.Md, r, nM, [&](int mode, double* acc) {
 #pragma unroll
       for (int v = 0; v < 5; ++v) acc[v] *= ep.scale;
       bad |= epilogue_mode(ep, nM, mode, acc);
@@ -729,7 +726,6 @@ __device__ __forceinline__ void element_ns_volume_t(const Ctx& c, const TypeTab&
   }
   // total contravariant flux G_l = sum_d M[l][d] (F_e - F_v)_d
   // (in place of the point's gradient)
-  fx_clear(fx_slots() + 10, 5);
   __syncthreads();
   auto put = [&](double* G, int v, double x) { G[v * nQ] = x; };
   for (int q = lane; q < nQ; q += blockDim.x) {
@@ -982,7 +978,7 @@ __device__ __forceinline__ void element_vjp_a_t(const Ctx& c, const VjpArgs& va,
   __syncthreads();
   if (dense) {
     const double* Md = cblk + 11 * nQ;
-    fx_dense(Md, bufC, nM, [&](int m, double* acc) {
+    dense_product(Md, bufC, nM, [&](int m, double* acc) {
 #pragma unroll
       for (int v = 0; v < 5; ++v) bufG[v * nM + m] = acc[v];
     });
@@ -1109,7 +1105,7 @@ __device__ __forceinline__ void element_vjp_a_ns_t(const Ctx& c, const VjpArgs& 
   __syncthreads();
   if (dense) {
     const double* Md = cblk + 11 * nQ;
-    fx_dense(Md, bufY, nM, [&](int m, double* acc) {
+    dense_product(Md, bufY, nM, [&](int m, double* acc) {
 #pragma unroll
       for (int v = 0; v < 5; ++v) bufS[v * nM + m] = acc[v];
     });

@@ -216,12 +216,6 @@ template <> struct FxTab<7> {
   static __device__ __forceinline__ int2 E(int end, int m) { return kFxE7[end * 7 + m]; }
 };
 
-// Exponent bookkeeping in shared memory: sets of five words (one per variable).
-__device__ __forceinline__ unsigned* fx_slots() {
-  __shared__ unsigned s[15];
-  return s;
-}
-
 struct FxD {
   int h, l;   // D = h 2^31 + l, 0 <= l < 2^31
 };
@@ -293,31 +287,6 @@ __device__ __forceinline__ unsigned fx_mag(long long R) {
 __device__ __forceinline__ long long fx_madw(int a, int b, long long c) { return (long long)a * b + c; }
 
 __device__ __forceinline__ unsigned fx_hi(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
-
-// Block maximum of every lane's five m[v] into slot[v] (zero before; a
-// barrier must follow).
-template <class I>
-__device__ __forceinline__ void fx_flush_max(const I* m, I* slot) {
-  const int l32 = threadIdx.x & 31;
-  I x = 0;
-#pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    const I r = __reduce_max_sync(0xffffffffu, m[v]);
-    x = l32 == v ? r : x;
-  }
-  if (l32 < 5) atomicMax(slot + l32, x);
-}
-
-// Largest high words of buf[v stride + i], i < cnt, into m[v]
-__device__ __forceinline__ void fx_scan(const double* buf, int cnt, int stride, unsigned* m) {
-#pragma unroll
-  for (int v = 0; v < 5; ++v)
-    for (int q = threadIdx.x; q < cnt; q += blockDim.x) m[v] = max(m[v], fx_hi(buf[v * stride + q]));
-}
-
-__device__ __forceinline__ void fx_clear(unsigned* slot, int cnt) {
-  for (int t = threadIdx.x; t < cnt; t += blockDim.x) slot[t] = 0u;
-}
 
 // Exponents of the lines between two passes: two sets of [5][n^2] lines, the
 // second also as [4][5][n] lines of face values
@@ -901,74 +870,26 @@ __device__ __forceinline__ void fx_lift(const TypeTab& T, LoadH H, const double*
   }
 }
 
-// out(mode, acc[5]) = Md r: Md [nM][nM] doubles in global memory, symmetric and
-// positive definite (its largest entry is on the diagonal), r [5][nM] doubles
-// in shared memory (destroyed).  Both become 54-bit integers (rounded) in two 27-bit
-// halves: the four products of a term and their sums over nM <= 196 terms fit
-// 64 bits, so nothing is dropped or shifted before the end.  A lane owns a
-// mode: one load and conversion of Md feeds five variables.  FP64 took 5
-// multiply-adds per entry, 94 clocks of the SM per warp; this is about 45
-// instructions, and what bounds it is the latency of Md's loads (two curved
-// 12^3 steps at N = 4: 4.13 -> 4.06 ms; an L2 prefetch of Md at the start of the
-// phase made it 4.14, unrolling by 8 4.20).
+// out(mode, acc[5]) = Md r: the dense inverse mass matrix of a curved element
+// (Algorithm 1 with a pointwise J), Md [nM][nM] in global memory, symmetric, r
+// [5][nM] in shared memory.  Lanes run over output modes, so the column reads of
+// Md are coalesced and every load feeds 5 sums.  In FP64: the modes of r and the
+// entries of a row of Md span many orders, and the small ones count in theirs.
+// What bounds it is the latency of Md's loads (two curved 12^3 steps at N = 4:
+// 4.01 ms; on integers with one exponent for all of r and one for Md 4.07).
 template <class Out>
-__device__ __forceinline__ void fx_dense(const double* Md, double* r, int nM, Out out) {
-  unsigned* sx = fx_slots();   // five words for r, one for Md
-  fx_clear(sx, 6);
-  __syncthreads();
-  unsigned m[5] = {0u, 0u, 0u, 0u, 0u}, md = 0u;
-  fx_scan(r, nM, nM, m);
-  for (int a = threadIdx.x; a < nM; a += blockDim.x) md = max(md, fx_hi(Md[(size_t)a * (nM + 1)]));
-  fx_flush_max(m, sx);
-  md = __reduce_max_sync(0xffffffffu, md);
-  if ((threadIdx.x & 31) == 0 && md) atomicMax(sx + 5, md);
-  __syncthreads();
-  constexpr int kLow = (1 << 27) - 1;
-  auto halves = [](long long D) {   // 55 bits -> 54, rounded
-    D = (D + 1) >> 1;
-    return make_int2((int)(D >> 27), (int)D & kLow);
-  };
-  int2* ri = reinterpret_cast<int2*>(r);
-#pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    const int em = fx_em(sx[v]) + 6;
-    for (int a = threadIdx.x; a < nM; a += blockDim.x) ri[v * nM + a] = halves(fx_from(r[v * nM + a], em));
-  }
-  __syncthreads();
-  const int emd = fx_em(sx[5]) + 6;
+__device__ __forceinline__ void dense_product(const double* Md, const double* r, int nM, Out out) {
   for (int a = threadIdx.x; a < nM; a += blockDim.x) {
-    long long hh[5], mid[5], ll[5];
-#pragma unroll
-    for (int v = 0; v < 5; ++v) hh[v] = mid[v] = ll[v] = 0;
+    const double* Mc = Md + a;
+    double acc[5] = {0, 0, 0, 0, 0};
 #pragma unroll 4
     for (int j = 0; j < nM; ++j) {
-      int2 k = halves(fx_from(Md[(size_t)j * nM + a], emd));
-      asm("" : "+r"(k.y));   // see fx_madw
+      const double m = Mc[(size_t)j * nM];
 #pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        int2 d = ri[v * nM + j];
-        asm("" : "+r"(d.y));
-        hh[v] = fx_madw(d.x, k.x, hh[v]);
-        mid[v] = fx_madw(d.x, k.y, mid[v]);
-        mid[v] = fx_madw(d.y, k.x, mid[v]);
-        ll[v] = fx_madw(d.y, k.y, ll[v]);
-      }
-    }
-    double acc[5];
-#pragma unroll
-    for (int v = 0; v < 5; ++v) {
-      // hh 2^54 + mid 2^27 + ll, |sum| < 2^116, as (hi, lo) = 2^27 hi + lo, then the top 64 bits
-      const long long t = mid[v] + (ll[v] >> 27);
-      const long long hi = hh[v] + (t >> 27);                    // units of 2^54
-      const unsigned lo = (unsigned)t & (unsigned)kLow;          // next 27 bits
-      const int ks = fx_shift(fx_mag(hi)), k = min(ks, 27);
-      const long long R = (hi << k) | (long long)(lo >> (27 - k));
-      // hi 2^54 units: value = hi 2^(54 - (1083 - em_r) - (1083 - em_d)); fx_to takes R 2^(eb - 1084)
-      acc[v] = fx_to(R, (fx_em(sx[v]) + 7) + (emd + 1) - 1028 - k);
+      for (int v = 0; v < 5; ++v) acc[v] = fma(m, r[v * nM + j], acc[v]);
     }
     out(a, acc);
   }
-  __syncthreads();
 }
 
 }  // namespace

@@ -37,8 +37,6 @@ static inline unsigned __funnelshift_r(unsigned lo, unsigned hi, unsigned s) { r
 static inline unsigned __funnelshift_l(unsigned lo, unsigned hi, unsigned s) { return (unsigned)(((((uint64_t)hi << 32) | lo) << (s & 31)) >> 32); }
 static inline int __clz(int x) { return x ? __builtin_clz((unsigned)x) : 32; }
 template <class T> static inline T __ldg(const T* p) { return *p; }
-template <class T> static inline T __reduce_max_sync(unsigned, T x) { return x; }
-template <class T> static inline void atomicMax(T* p, T x) { *p = max(*p, x); }
 static inline void __syncthreads() {}
 static inline int __syncthreads_or(int x) { return x; }
 #include "dg_fixed.cuh"
@@ -110,6 +108,11 @@ int t_lift_modal(int n, int type, const double* H, const double* F, int neg, int
 }
 int t_nodal(int n, int type, const double* Q, double* out, double* tr) { return EACH(n, nodal)(type, Q, out, tr); }
 int t_modal(int n, int type, const double* U, double* out) { return EACH(n, modal)(type, U, out); }
+void t_dense(int nM, const double* Md, const double* r, double* out) {
+  dense_product(Md, r, nM, [&](int a, const double* acc) {
+    for (int v = 0; v < 5; ++v) out[v * nM + a] = acc[v];
+  });
+}
 void t_grad(int n, const double* U, double* out) { EACH(n, grad)(U, out); }
 // nodes, Lagrange end values, and the factors of the basis at the nodes
 int t_tables(int n, int type, double* A, double* V, double* ext, int* face) {

@@ -95,3 +95,16 @@ def test_lift_to_modal_keeps_line_scales(fx, n, etype):  # noqa: F811
             out = np.empty((5, nM))
             assert fx.t_lift_modal(n, etype, ptr(H), ptr(F), neg, stage, ptr(out)) == nM
             assert (np.abs(out - ref) <= bound).all()
+
+
+@pytest.mark.parametrize("nM", [4, 18, 75])
+def test_dense_product_keeps_small_modes(fx, nM):  # noqa: F811
+    """A mildly bent element's inverse mass matrix on modes that decay over twelve orders."""
+    rng = np.random.default_rng(nM)
+    M = rng.uniform(-1, 1, (nM, nM)) * 1e-6
+    M = np.diag(rng.uniform(0.5, 2, nM)) + M + M.T
+    r = rng.uniform(-1, 1, (5, nM)) * 10.0 ** np.linspace(0, -12, nM)
+    out = np.empty((5, nM))
+    fx.t_dense(nM, ptr(M), ptr(r), ptr(out))
+    ref = r.astype(LD) @ M.astype(LD)
+    assert (np.abs(out - ref) <= (nM + 3) * U * (np.abs(r) @ np.abs(M))).all()
