@@ -61,15 +61,18 @@ constexpr int kSplitBlocks = kn <= 3 ? 6 : (kn == 4 ? 4 : 5);
   } while (0)
 
 // Modal -> nodal by the sum-factorised passes: sQ [5][nM] (modal
-// coefficients) -> U in bufA [5][nQ]; bufB is scratch (sQ may alias it).
+// coefficients) -> U in bufA [5][nQ]; bufB is scratch (sQ may alias it).  IEEE:
+// the one-shot maps (fx_wild).
+template <bool IEEE>
 __device__ __forceinline__ void modal_to_nodal_passes(const Ctx& c, const TypeTab& T, const double* sQ, double* bufA,
                                                       double* bufB) {
-  fx_to_nodal<kn, false>(c, T, sQ, bufA, bufB, [](int, int, int, double) {});
+  fx_to_nodal<kn, false, IEEE>(c, T, sQ, bufA, bufB, [](int, int, int, double) {});
 }
 
 // Storage -> nodal: U = V Q in bufA [5][nQ] from a stored element block sQ.
 // A hexahedron is stored as s = W^{1/2} V Q, so U = W^{-1/2} s pointwise;
 // the other types hold modal coefficients.  sQ may alias bufB.
+template <bool IEEE = false>
 __device__ __forceinline__ void modal_to_nodal(const Ctx& c, const TypeTab& T, const double* sQ, double* bufA,
                                             double* bufB, int lane) {
   if (T.type == HEX) {
@@ -79,7 +82,7 @@ __device__ __forceinline__ void modal_to_nodal(const Ctx& c, const TypeTab& T, c
     __syncthreads();
     return;
   }
-  modal_to_nodal_passes(c, T, sQ, bufA, bufB);
+  modal_to_nodal_passes<IEEE>(c, T, sQ, bufA, bufB);
 }
 
 // What the nodal->modal pass does with r = M_ref^{-1} V^T bufA of a mode
@@ -165,7 +168,7 @@ __device__ __forceinline__ bool finish_modal(const Ctx& c, const TypeTab& T, dou
 
 // Nodal -> modal transpose: bufA [5][nQ] -> modal coefficients through `ep`;
 // bufB is scratch.  Returns true if a non-finite state value was produced.
-template <bool DENSE>
+template <bool DENSE, bool IEEE = false>
 __device__ __forceinline__ bool nodal_to_modal_t(const Ctx& c, const TypeTab& T, double* bufA, double* bufB, int lane,
                                               const Epilogue& ep) {
   constexpr int nQ = knQ;
@@ -186,17 +189,17 @@ __device__ __forceinline__ bool nodal_to_modal_t(const Ctx& c, const TypeTab& T,
     return bad;
   }
   double* r = DENSE ? ep.rbuf : bufB;
-  fx_to_modal<kn>(T, c, bufA, bufB, r);
+  fx_to_modal<kn, IEEE>(T, c, bufA, bufB, r);
   return finish_modal<DENSE>(c, T, r, lane, ep);
 }
 
 // ANY: the launch may meet curved elements (their variants are compiled into
 // the kernel only then, so affine launches keep the affine register budget).
-template <bool ANY>
+template <bool ANY, bool IEEE = false>
 __device__ __forceinline__ bool nodal_to_modal(const Ctx& c, const TypeTab& T, double* bufA, double* bufB, int lane,
                                                const Epilogue& ep) {
-  return (ANY && ep.Md) ? nodal_to_modal_t<true>(c, T, bufA, bufB, lane, ep)
-                        : nodal_to_modal_t<false>(c, T, bufA, bufB, lane, ep);
+  return (ANY && ep.Md) ? nodal_to_modal_t<true, IEEE>(c, T, bufA, bufB, lane, ep)
+                        : nodal_to_modal_t<false, IEEE>(c, T, bufA, bufB, lane, ep);
 }
 
 // Values of the nodal field `src` [5][nQ] on the element's own face points
@@ -440,7 +443,7 @@ __device__ __forceinline__ void element_forward_t(const Ctx& c, const TypeTab& T
     write_traces(c, T, s, bufA, c.T);
   } else {
     const int64_t* ft = c.slot_ftoff + s * 6;
-    fx_to_nodal<kn, true>(c, T, bufG, bufA, bufG,
+    fx_to_nodal<kn, true, false>(c, T, bufG, bufA, bufG,
                           [&](int lf, int v, int p, double x) { c.T[__ldg(ft + lf) + v * kn2 + p] = x; });
   }
   if (c.Usave) {
@@ -635,7 +638,7 @@ __device__ __forceinline__ void element_ns_volume_t(const Ctx& c, const TypeTab&
       for (int w = lane; w < 5 * T.nM; w += blockDim.x) sG[w] = Gm[w];
       __syncthreads();
       const int64_t* ft = c.slot_ftoff + s * 6;
-      fx_to_nodal<kn, true>(c, T, sG, dW, bufG, [&](int lf, int v, int p, double x) {
+      fx_to_nodal<kn, true, false>(c, T, sG, dW, bufG, [&](int lf, int v, int p, double x) {
         c.Vt[3 * __ldg(ft + lf) + (d * 5 + v) * n2 + p] = x;
       });
     }
@@ -712,7 +715,7 @@ __device__ __forceinline__ void element_ns_volume_t(const Ctx& c, const TypeTab&
       Epilogue ep{Epilogue::kStore, true, CURVED ? -1.0 : -g.invJ, sG, nullptr, nullptr, nullptr, nullptr, 0.0, 0.0};
       if (CURVED) ep.Md = cblk + 11 * nQ;
       finish_modal<CURVED>(c, T, bufA, lane, ep);
-      fx_to_nodal<kn, true>(c, T, sG, dW, bufG, [&](int lf, int v, int p, double x) {
+      fx_to_nodal<kn, true, false>(c, T, sG, dW, bufG, [&](int lf, int v, int p, double x) {
         c.Vt[3 * __ldg(ft + lf) + (d * 5 + v) * n2 + p] = x;
       });
     }
@@ -803,7 +806,7 @@ __device__ __forceinline__ void process_element(const Ctx& c, int mode, const St
     const double* Q = io.Qin + c.elem_qoff[c.elem_of_slot[s]];
     for (int w = lane; w < 5 * nM; w += blockDim.x) bufG[w] = Q[w];
     __syncthreads();
-    modal_to_nodal_passes(c, T, bufG, bufA, bufG);
+    modal_to_nodal_passes<true>(c, T, bufG, bufA, bufG);
     const double* sq = c.dpool + T.sqw;
     double* out = io.Qout + qoff;
     for (int w = lane; w < 5 * nQ; w += blockDim.x) out[w] = bufA[w] * sq[w % nQ];
@@ -819,7 +822,7 @@ __device__ __forceinline__ void process_element(const Ctx& c, int mode, const St
     Epilogue ep{Epilogue::kStore, false, 1.0, io.Qout + c.elem_qoff[c.elem_of_slot[s]], nullptr, nullptr, nullptr,
                 nullptr, 0.0, 0.0};
     ep.modal = true;
-    nodal_to_modal_t<false>(c, T, bufA, bufG, lane, ep);
+    nodal_to_modal_t<false, true>(c, T, bufA, bufG, lane, ep);
     return;
   }
   if constexpr (FAM == kStage) if (mode == kFwd) {
@@ -853,7 +856,7 @@ __device__ __forceinline__ void process_element(const Ctx& c, int mode, const St
     const double* Q = io.Qin + qoff;
     for (int w = lane; w < 5 * nM; w += blockDim.x) bufG[w] = Q[w];
     __syncthreads();
-    modal_to_nodal(c, T, bufG, bufA, bufG, lane);
+    modal_to_nodal<true>(c, T, bufG, bufA, bufG, lane);
     double* out = io.Qout + c.elem_voff[c.elem_of_slot[s]];
     for (int w = lane; w < 5 * nQ; w += blockDim.x) out[w] = bufA[w];
     __syncthreads();
@@ -883,7 +886,7 @@ __device__ __forceinline__ void process_element(const Ctx& c, int mode, const St
     __syncthreads();
     Epilogue ep{Epilogue::kStore, false, cblk ? 1.0 : 1.0 / c.geo[s].invJ, io.Qout + qoff, nullptr, nullptr, nullptr,
                 nullptr, 0.0, 0.0};
-    nodal_to_modal<false>(c, T, bufA, bufG, lane, ep);
+    nodal_to_modal<false, true>(c, T, bufA, bufG, lane, ep);
     return;
   }
   if constexpr (FAM == kMisc) if (mode == kProject) {
@@ -902,7 +905,7 @@ __device__ __forceinline__ void process_element(const Ctx& c, int mode, const St
       ep.Md = cblk + 11 * nQ;
       ep.rbuf = bufG + 5 * nQ;
     }
-    nodal_to_modal<ANY>(c, T, bufA, bufG, lane, ep);
+    nodal_to_modal<ANY, true>(c, T, bufA, bufG, lane, ep);
     return;
   }
   if constexpr (FAM == kStage) {
@@ -1433,7 +1436,7 @@ __device__ void mass_product(const Ctx& c, const TypeTab& T, const double* x, co
                              double* r, double* bufA, double* bufB, int tid) {
   constexpr int nQ = knQ;
   const int nM = T.nM;
-  modal_to_nodal_passes(c, T, x, bufA, bufB);
+  modal_to_nodal_passes<false>(c, T, x, bufA, bufB);
   for (int w = tid; w < 5 * nQ; w += blockDim.x) bufA[w] *= wJ[w % nQ];
   __syncthreads();
   Epilogue ep{Epilogue::kStore, false, 1.0, r, nullptr, nullptr, nullptr, nullptr, 0.0, 0.0};

@@ -7,12 +7,12 @@
 // the coefficients are 62-bit integers C = ch 2^31 + cl, and
 //   sum C D / 2^62 = sum dh ch + (sum dh cl + dl ch) / 2^31
 // takes three multiply-adds per term (the dl cl products lie below the last
-// bit kept).  The last bit is 2^-61 of the largest input times the row's
-// growth, against 2^-53 of every partial sum in FP64, and the result is
-// rounded once, to nearest, when it becomes a double again; so the
-// contraction is as accurate as the FP64 chain or better for every input
-// whose block is finite.  A block that holds an infinity or a NaN gives NaN
-// throughout, zeros give zeros, and results below the normal range give zero.
+// bit kept), and the result is rounded once, to nearest, when it becomes a
+// double again.  Its error is at most 2^(g - 58) of the line's largest value,
+// with 2^g above the row's sum of |c|: FP64's own for a row that counts that
+// value.  A row that does not (the zero coefficients of the middle node, n odd;
+// the ragged passes' near the degenerate edge) keeps less beside it than FP64.
+// For infinities, NaNs and subnormals see fx_wild.
 //
 // A value keeps its scale as `eb`: |x| < 2^(eb - 1023), x = R 2^(eb - 1084).
 // Between the passes of one transform the integers stay in shared memory,
@@ -230,12 +230,12 @@ __device__ __forceinline__ FxD fx_split(long long D, int k) {
   return f;
 }
 
-// x 2^(1083 - em) as an integer, |x| < 2^(em + 1 - 1023); neg: of -x.  A
-// subnormal x counts half (its exponent field is that of no hidden bit).
+// x 2^(1083 - em) as an integer, |x| < 2^(em + 1 - 1023), em > 0; neg: of -x.
 __device__ __forceinline__ long long fx_from(double x, int em, unsigned neg = 0u) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), e = (hi >> 20) & 0x7ffu;
-  const int d = min(em - (int)e, 63);
-  const unsigned mh = (__funnelshift_l(lo, hi, 8) & 0x0fffffffu) | (min(e, 1u) << 28), ml = lo << 8;
+  const unsigned b = min(e, 1u);   // a subnormal has no hidden bit and the exponent of field 1
+  const int d = min(em - 1 + (int)b - (int)e, 63);
+  const unsigned mh = (__funnelshift_l(lo, hi, 8) & 0x0fffffffu) | (b << 28), ml = lo << 8;
   const unsigned long long M = (((unsigned long long)mh << 32) | ml) >> d;
   const long long s = (long long)((int)(hi ^ neg) >> 31);
   return ((long long)M ^ s) - s;
@@ -268,8 +268,15 @@ __device__ __forceinline__ double fx_to(long long R, int eb) {
 // exponent of a block from the largest high word (sign cleared) of its values
 __device__ __forceinline__ int fx_em(unsigned hmax) {
   const int e = (int)(hmax >> 20);
-  return e == 2047 ? kFxBad + 2047 : e;
+  return e == 2047 ? kFxBad + 2047 : max(e, 1);
 }
+
+// Whether the largest high word of a line is outside [2^-963, 2^1006) and not
+// zero: infinities, NaNs, subnormals and what comes near them.  The phases of a
+// residual give NaN for what meets an infinity or a NaN and zero below the normal
+// range; the one-shot maps, whose results are the caller's, compute such an
+// element in FP64 (the fx_..._ieee functions): infinities by value, subnormals.
+__device__ __forceinline__ bool fx_wild(unsigned hmax) { return hmax - 0x03c00000u > 0x7b000000u && hmax != 0u; }
 
 // shift that brings integers with OR of high words (one's complement) m to 61 bits
 __device__ __forceinline__ int fx_shift(unsigned m) { return max(__clz((int)m) - 3, 0); }
@@ -339,6 +346,14 @@ __device__ __forceinline__ long long fx_dot(const FxD* d, Coef C, long long mid 
 #pragma unroll
   for (int m = 0; m < n; ++m) hh = fx_madw(d[m].h, C(m).x, hh);
   return hh;
+}
+
+template <int n>
+__device__ __forceinline__ bool fx_wild_line(const double* x) {
+  bool w = false;
+#pragma unroll
+  for (int i = 0; i < n; ++i) w |= fx_wild(fx_hi(x[i]));
+  return w;
 }
 
 // Exponent of n doubles (their largest) and their integers
@@ -417,12 +432,85 @@ __device__ __forceinline__ void fx_traces(const TypeTab& T, const double* src, O
   }
 }
 
+// The transforms in FP64, for elements the integers do not hold (fx_wild): the
+// sum-factorised passes, one output per lane at a time.
+template <int n>
+__device__ __forceinline__ void fx_nodal_ieee(const Ctx& c, const TypeTab& T, const double* sQ, double* bufA, double* bufB) {
+  constexpr int n2 = n * n, nQ = n2 * n;
+  const double* dp = c.dpool;
+  const int* ip = c.ipool;
+  const int nM = T.nM, cn = T.ncols * n;
+  for (int o = threadIdx.x; o < 5 * cn; o += blockDim.x) {
+    const int v = o / cn, r = o - v * cn, col = r / n;
+    const double* C = dp + T.C + ip[T.col_coff + col] + r - col * n;
+    const double* q = sQ + v * nM + ip[T.col_moff + col];
+    double acc = 0.0;
+#pragma unroll 1
+    for (int t = 0; t < ip[T.col_len + col]; ++t) acc = fma(C[t * n], q[t], acc);
+    bufA[v * nQ + r] = acc;
+  }
+  __syncthreads();
+  for (int o = threadIdx.x; o < 5 * nQ; o += blockDim.x) {
+    const int v = o / nQ, r = o - v * nQ, p = r / n2, j = r / n % n, k = r % n;
+    const double* B = dp + T.B + ip[T.p_boff + p] + j;
+    const double* X = bufA + v * nQ + ip[T.p_cbase + p] * n + k;
+    double acc = 0.0;
+#pragma unroll 1
+    for (int t = 0; t < ip[T.p_blen + p]; ++t) acc = fma(B[t * n], X[t * n], acc);
+    bufB[o] = acc;
+  }
+  __syncthreads();
+  for (int o = threadIdx.x; o < 5 * nQ; o += blockDim.x) {
+    const int v = o / nQ, r = o - v * nQ, i = r / n2;
+    double acc = 0.0;
+#pragma unroll 1
+    for (int p = 0; p < n; ++p) acc = fma(dp[T.A + p * n + i], bufB[v * nQ + p * n2 + r % n2], acc);
+    bufA[o] = acc;
+  }
+  __syncthreads();
+}
+
+// bufA [5][nQ] (destroyed) -> r [5][nM]; r may alias bufB, not bufA
+template <int n>
+__device__ __forceinline__ void fx_modal_ieee(const Ctx& c, const TypeTab& T, double* bufA, double* bufB, double* r) {
+  constexpr int n2 = n * n, nQ = n2 * n;
+  const double* dp = c.dpool;
+  const int* ip = c.ipool;
+  const int nM = T.nM, cn = T.ncols * n;
+  for (int o = threadIdx.x; o < 5 * nQ; o += blockDim.x) {
+    const int v = o / nQ, w = o - v * nQ, p = w / n2;
+    double acc = 0.0;
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) acc = fma(dp[T.A + p * n + i], bufA[v * nQ + i * n2 + w % n2], acc);
+    bufB[o] = acc;
+  }
+  __syncthreads();
+  for (int o = threadIdx.x; o < 5 * cn; o += blockDim.x) {
+    const int v = o / cn, w = o - v * cn, col = w / n, p = ip[T.col_p + col];
+    const double* B = dp + T.B + ip[T.p_boff + p] + (col - ip[T.p_cbase + p]) * n;
+    double acc = 0.0;
+#pragma unroll 1
+    for (int j = 0; j < n; ++j) acc = fma(B[j], bufB[v * nQ + p * n2 + j * n + w % n], acc);
+    bufA[v * nQ + w] = acc;
+  }
+  __syncthreads();
+  for (int o = threadIdx.x; o < 5 * nM; o += blockDim.x) {
+    const int v = o / nM, mode = o - v * nM, col = ip[T.mode_col + mode];
+    const double* C = dp + T.C + ip[T.col_coff + col] + (mode - ip[T.col_moff + col]) * n;
+    double acc = 0.0;
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) acc = fma(C[k], bufA[v * nQ + col * n + k], acc);
+    r[o] = acc;
+  }
+  __syncthreads();
+}
+
 // Modal -> nodal, U = V Q: sQ [5][nM] doubles -> bufA [5][nQ] doubles, bufB
 // [5][nQ] scratch (sQ may alias bufB).  Passes c, b, a, one line per lane.
 // TR: the values at the element's face points too, out(local face, variable,
 // face point, value), bit for bit fx_traces of U (the a faces by the lane that
-// forms the line).
-template <int n, bool TR, class Out>
+// forms the line).  IEEE: an element of fx_wild's range goes through FP64.
+template <int n, bool TR, bool IEEE, class Out>
 __device__ __forceinline__ void fx_to_nodal(const Ctx& c, const TypeTab& T, const double* sQ, double* bufA,
                                             double* bufB, Out out) {
   constexpr int n2 = n * n, nQ = n2 * n;
@@ -434,6 +522,7 @@ __device__ __forceinline__ void fx_to_nodal(const Ctx& c, const TypeTab& T, cons
   long long* X = reinterpret_cast<long long*>(bufA);
   long long* Y = reinterpret_cast<long long*>(bufB);
   const bool uc = T.type == HEX || T.type == PRISM, ub = T.type == HEX || T.type == PYR;
+  unsigned wild = 0u;
   // c-pass: X[col][k] = sum_t C[col][t][k] Q[moff[col] + t]
   for (int t0 = threadIdx.x; t0 < 5 * ncols; t0 += nt) {
     const int v = t0 / ncols, col = t0 - v * ncols;
@@ -444,6 +533,7 @@ __device__ __forceinline__ void fx_to_nodal(const Ctx& c, const TypeTab& T, cons
       double x[n];
 #pragma unroll
       for (int t = 0; t < n; ++t) x[t] = q[t];
+      if (IEEE) wild |= fx_wild_line<n>(x);
       FxD d[n];
       eb = fx_line<n>(x, d) + 1 + Tab::gA;
 #pragma unroll
@@ -454,13 +544,23 @@ __device__ __forceinline__ void fx_to_nodal(const Ctx& c, const TypeTab& T, cons
       const int* ms = ip + T.mode_s + (q - sQ - v * nM);
       int em = fx_em(fx_hi(q[0])) + __ldg(ms);
       for (int t = 1; t < len; ++t) em = max(em, fx_em(fx_hi(q[t])) + __ldg(ms + t));
+      if (IEEE)
+        for (int t = 0; t < len; ++t) wild |= fx_wild(fx_hi(q[t]));
       eb = em + 1 + kFxGR;
       fx_ragged_out<n>(c.fpool + T.C + __ldg(ip + T.col_coff + col), len,
                        [&](int t) { return fx_split(fx_from(q[t], em - __ldg(ms + t)), 0); }, R);
     }
     e0[v * n2 + col] = fx_store_line<n>(R, eb, X + v * nQ + col * n, 1);
   }
-  __syncthreads();
+  if (IEEE) {
+    static_assert(!(TR && IEEE), "the one-shot maps take no traces");
+    if (__syncthreads_or(wild)) {
+      fx_nodal_ieee<n>(c, T, sQ, bufA, bufB);
+      return;
+    }
+  } else {
+    __syncthreads();
+  }
   // b-pass: Y[p][j][k] = sum_t B[p][t][j] X[cbase[p] + t][k]
   for (int t0 = threadIdx.x; t0 < 5 * n2; t0 += nt) {
     const int v = t0 / n2, pk = t0 - v * n2, p = pk / n, k = pk - p * n;
@@ -574,12 +674,13 @@ __device__ __forceinline__ void fx_modal_tail(const Ctx& c, const TypeTab& T, co
 
 // Nodal -> modal transpose, r = V^T h: bufA [5][nQ] doubles (destroyed) ->
 // r [5][nM] doubles; bufB [5][nQ] scratch (r may alias bufB, not bufA).
-template <int n>
+template <int n, bool IEEE>
 __device__ __forceinline__ void fx_to_modal(const TypeTab& T, const Ctx& c, double* bufA, double* bufB, double* r) {
   constexpr int n2 = n * n, nQ = n2 * n;
   using Tab = FxTab<n>;
   int* e0 = fx_exps<n>();
   long long* Y = reinterpret_cast<long long*>(bufB);
+  unsigned wild = 0u;
   // a-pass: Y[p][j][k] = sum_i A[p][i] h[i][j][k]
   for (int t0 = threadIdx.x; t0 < 5 * n2; t0 += blockDim.x) {
     const int v = t0 / n2, jk = t0 - v * n2;
@@ -587,6 +688,7 @@ __device__ __forceinline__ void fx_to_modal(const TypeTab& T, const Ctx& c, doub
     double x[n];
 #pragma unroll
     for (int i = 0; i < n; ++i) x[i] = h[i * n2];
+    if (IEEE) wild |= fx_wild_line<n>(x);
     FxD d[n];
     const int eb = fx_line<n>(x, d) + 1 + Tab::gA;
     long long R[n];
@@ -594,7 +696,14 @@ __device__ __forceinline__ void fx_to_modal(const TypeTab& T, const Ctx& c, doub
     for (int p = 0; p < n; ++p) R[p] = fx_dot<n>(d, [&](int i) { return Tab::A(p, i); });
     e0[v * n2 + jk] = fx_store_line<n>(R, eb, Y + v * nQ + jk, n2);
   }
-  __syncthreads();
+  if (IEEE) {
+    if (__syncthreads_or(wild)) {
+      fx_modal_ieee<n>(c, T, bufA, bufB, r);
+      return;
+    }
+  } else {
+    __syncthreads();
+  }
   fx_modal_tail<n>(c, T, Y, reinterpret_cast<long long*>(bufA), r);
 }
 
@@ -876,7 +985,8 @@ __device__ __forceinline__ void fx_lift(const TypeTab& T, LoadH H, const double*
 // Md are coalesced and every load feeds 5 sums.  In FP64: the modes of r and the
 // entries of a row of Md span many orders, and the small ones count in theirs.
 // What bounds it is the latency of Md's loads (two curved 12^3 steps at N = 4:
-// 4.01 ms; on integers with one exponent for all of r and one for Md 4.07).
+// 3.95 ms; 4.02 on integers with one exponent for all of r and one for Md, which
+// left modes that decay over twelve orders 1e-8 of themselves off).
 template <class Out>
 __device__ __forceinline__ void dense_product(const double* Md, const double* r, int nM, Out out) {
   for (int a = threadIdx.x; a < nM; a += blockDim.x) {

@@ -79,35 +79,40 @@ template <int n> int lift_modal(int type, const double* H, const double* F, int 
   memcpy(out, stage ? A : G + m, 5 * s.T.nM * sizeof(double));
   return s.T.nM;
 }
-template <int n> int nodal(int type, const double* Q, double* out, double* tr) {
+template <int n, bool IEEE> int nodal(int type, const double* Q, double* out, double* tr) {
   constexpr int n2 = n * n, m = 5 * n * n2;
   Setup s(type, n - 1);
   double A[m], B[m];
   memcpy(B, Q, 5 * s.T.nM * sizeof(double));
-  fx_to_nodal<n, true>(s.c, s.T, B, A, B, [&](int lf, int v, int p, double x) { tr[(lf * 5 + v) * n2 + p] = x; });
+  fx_to_nodal<n, !IEEE, IEEE>(s.c, s.T, B, A, B, [&](int lf, int v, int p, double x) { tr[(lf * 5 + v) * n2 + p] = x; });
   memcpy(out, A, sizeof(A));
   return s.T.nM;
 }
-template <int n> int modal(int type, const double* U, double* out) {
+template <int n, bool IEEE> int modal(int type, const double* U, double* out) {
   constexpr int m = 5 * n * n * n;
   Setup s(type, n - 1);
   double A[m], B[m];
   memcpy(A, U, sizeof(A));
-  fx_to_modal<n>(s.T, s.c, A, B, B);
+  fx_to_modal<n, IEEE>(s.T, s.c, A, B, B);
   memcpy(out, B, 5 * s.T.nM * sizeof(double));
   return s.T.nM;
 }
 template <int n> void grad(const double* U, double* out) { fx_grad<n>(U, out); }
 }  // namespace
 #define EACH(n, f) (n == 2 ? f<2> : n == 3 ? f<3> : n == 4 ? f<4> : n == 5 ? f<5> : n == 6 ? f<6> : f<7>)
+#define EACH2(n, f, b) (n == 2 ? f<2, b> : n == 3 ? f<3, b> : n == 4 ? f<4, b> : n == 5 ? f<5, b> : n == 6 ? f<6, b> : f<7, b>)
 extern "C" {
 void t_dsum(int n, const double* G, unsigned dirs, double* out) { EACH(n, dsum)(G, dirs, out); }
 void t_lift(int n, int type, const double* H, const double* F, int neg, double* out) { EACH(n, lift)(type, H, F, neg, out); }
 int t_lift_modal(int n, int type, const double* H, const double* F, int neg, int stage, double* out) {
   return EACH(n, lift_modal)(type, H, F, neg, stage, out);
 }
-int t_nodal(int n, int type, const double* Q, double* out, double* tr) { return EACH(n, nodal)(type, Q, out, tr); }
-int t_modal(int n, int type, const double* U, double* out) { return EACH(n, modal)(type, U, out); }
+int t_nodal(int n, int type, int ieee, const double* Q, double* out, double* tr) {
+  return ieee ? EACH2(n, nodal, true)(type, Q, out, tr) : EACH2(n, nodal, false)(type, Q, out, tr);
+}
+int t_modal(int n, int type, int ieee, const double* U, double* out) {
+  return ieee ? EACH2(n, modal, true)(type, U, out) : EACH2(n, modal, false)(type, U, out);
+}
 void t_dense(int nM, const double* Md, const double* r, double* out) {
   dense_product(Md, r, nM, [&](int a, const double* acc) {
     for (int v = 0; v < 5; ++v) out[v * nM + a] = acc[v];

@@ -108,3 +108,82 @@ def test_dense_product_keeps_small_modes(fx, nM):  # noqa: F811
     fx.t_dense(nM, ptr(M), ptr(r), ptr(out))
     ref = r.astype(LD) @ M.astype(LD)
     assert (np.abs(out - ref) <= (nM + 3) * U * (np.abs(r) @ np.abs(M))).all()
+
+
+def kinds(a):
+    """0 finite, 1 +infinity, 2 -infinity, 3 NaN"""
+    return np.where(np.isnan(a), 3, np.where(np.isposinf(a), 1, np.where(np.isneginf(a), 2, 0)))
+
+
+@pytest.mark.parametrize("n", DEGREES)
+@pytest.mark.parametrize("etype", range(4))
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan, 1e303, 3e-310])
+def test_extreme_values(fx, n, etype, value):  # noqa: F811
+    """One infinity, NaN or huge value, or a variable of subnormals.  The one-shot maps give the FP64 sums:
+    infinities by value, gradual underflow.  The phases of a residual are not finite exactly where the FP64 sums
+    are not (NaN there), and lose what lies below the normal range."""
+    rng = np.random.default_rng(100 * n + etype)
+    V, face = tables(fx, n, etype)
+    D, E = (m.astype(float) for m in nodes(n)[1:])
+    nf, nM = face.max() + 1, V.shape[1]
+
+    def field(*shape):
+        a = rng.uniform(-1, 1, shape)
+        if value == 3e-310:
+            a[0] *= value
+        else:
+            a[0].flat[rng.integers(a[0].size)] = value
+        return a
+
+    def check(got, terms, ieee=False):
+        """terms: the products to be summed, along the last axis"""
+        size = np.abs(np.where(np.isfinite(terms), terms, 0)).sum(-1)
+        ref = terms.sum(-1)
+        if ieee:
+            assert (kinds(got) == kinds(ref)).all()
+        else:
+            assert (np.isnan(got) == ~np.isfinite(ref)).all() and not np.isinf(got).any()
+        ok = np.isfinite(ref)
+        if value == 1e303 and not ieee:
+            return            # the accuracy beside a large value: the tests above
+        # chains of three passes; 400 last bits of subnormals, or the end of the normal range
+        tiny = 400 * 2.0 ** -1074 if ieee else 2.0 ** -1022
+        assert (np.abs(got - ref)[ok] <= (6 * n + 20) * U * size[ok] + tiny).all()
+
+    with np.errstate(all="ignore"):
+        Q, W = field(5, nM), field(5, n, n, n)
+        A, R, tr = np.empty((5, n ** 3)), np.empty((5, nM)), np.empty((nf, 5, n, n))
+        for ieee in (0, 1):
+            fx.t_nodal(n, etype, ieee, ptr(Q), ptr(A), ptr(tr))
+            check(A, Q[:, None, :] * V[None], ieee)
+            fx.t_modal(n, etype, ieee, ptr(W), ptr(R))
+            check(R, W.reshape(5, -1)[:, None, :] * V.T[None], ieee)
+        g = np.empty((3, 5, n, n, n))
+        fx.t_grad(n, ptr(W), ptr(g))
+        for l in range(3):
+            check(along(g[l], l), along(W, l)[..., None, :] * D)
+        G = rng.uniform(-1, 1, (3, 5, n, n, n))
+        G[int(rng.integers(3))] = W
+        out = np.empty((5, n, n, n))
+        fx.t_dsum(n, ptr(G), 7, ptr(out))
+        check(out, np.concatenate([np.moveaxis(along(G[l], l)[..., None, :] * D.T, -2, 1 + l) for l in range(3)], axis=-1))
+        # the lift, of an extreme node or an extreme face value
+        for H, F in ((W, rng.uniform(-1, 1, (nf, 5, n, n))), (rng.uniform(-1, 1, W.shape), field(5, nf, n, n).swapaxes(0, 1).copy())):
+            if value == 3e-310:
+                H, F = H * 1.0, F * 1.0
+                H[0] = rng.uniform(-1, 1, H[0].shape) * value
+                F[:, 0] = rng.uniform(-1, 1, F[:, 0].shape) * value
+            terms = [H]
+            for k in range(6):
+                if face[k] >= 0:
+                    shape = [1, 1, 1, 1]
+                    shape[1 + k // 2] = n
+                    f = np.expand_dims(np.swapaxes(F[face[k]], 1, 2), 1 + k // 2)
+                    terms.append(np.broadcast_to(-E[k % 2].reshape(shape) * f, H.shape))
+            terms = np.stack(terms, axis=-1)
+            fx.t_lift(n, etype, ptr(H), ptr(F), 1, ptr(out))
+            check(out, terms)
+            both = (terms.reshape(5, 1, n ** 3, -1) * V.T[None, :, :, None]).reshape(5, nM, -1)
+            for stage in (0, 1):
+                fx.t_lift_modal(n, etype, ptr(H), ptr(F), 1, stage, ptr(R))
+                check(R, both)
