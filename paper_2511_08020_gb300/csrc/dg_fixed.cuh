@@ -356,6 +356,15 @@ __device__ __forceinline__ bool fx_wild_line(const double* x) {
   return w;
 }
 
+// a + b on the larger of their exponents (returned in e), the other rounded to
+// nearest: floors would lean every sum the same way (see S above).
+__device__ __forceinline__ long long fx_sum(long long a, int ea, long long b, int eb, int& e) {
+  const bool up = ea >= eb;
+  const int k = min(up ? ea - eb : eb - ea, 61);
+  e = up ? ea : eb;
+  return (up ? a : b) + (((up ? b : a) + ((1ll << k) >> 1)) >> k);
+}
+
 // Exponent of n doubles (their largest) and their integers
 template <int n>
 __device__ __forceinline__ int fx_line(const double* x, FxD* d) {
@@ -839,7 +848,8 @@ __device__ __forceinline__ void fx_dsum(Load load, unsigned dirs, double* tmp, d
   for (int l = 2; l >= 0; --l) {
     if (!((dirs >> l) & 1u)) continue;
     const bool last = (dirs & ((1u << l) - 1u)) == 0u;
-    // exponent of the sum so far at point m of a line: max(ea[m sa], eb[m sb]) + room
+    // exponent of the sum so far at point m of a line: the largest of its lines';
+    // a line's results are below 2^61, three of them below 2^63
     const bool two = l == 0 && (dirs & 6u) == 6u;
     const bool by1 = l == 0 && !(dirs & 4u);
     for (int t0 = threadIdx.x; t0 < 5 * n2; t0 += blockDim.x) {
@@ -869,8 +879,8 @@ __device__ __forceinline__ void fx_dsum(Load load, unsigned dirs, double* tmp, d
 #pragma unroll kUnroll
         for (int i = 0; i < n; ++i) {
           const long long R = fx_dot<n>(d, [&](int m) { return Tab::D(i, m); }, Tab::S(i));
-          const int ep = max(p[i * se], q[i * se]) + (two ? 1 : 0), e = max(ep, eb) + 1;
-          const long long r = (A[o + i * sd] >> min(e - ep, 63)) + (R >> min(e - eb, 63));
+          int e;
+          const long long r = fx_sum(A[o + i * sd], max(p[i * se], q[i * se]), R, eb, e);
           if (last) out[o + i * sd] = fx_to(r, e);
           else A[o + i * sd] = r;
         }
@@ -965,12 +975,15 @@ __device__ __forceinline__ void fx_lift(const TypeTab& T, LoadH H, const double*
         if (l == 2) {
           a = R;
         } else if (l == 1) {
-          const int ep = e2[i], e = max(ep, eb);
-          a = (a >> min(e - ep, 63)) + (R >> min(e - eb, 63));
+          int e;
+          a = fx_sum(a, e2[i], R, eb, e);
         } else {
           const double h = H(o + i * sd);
-          const int ep = max(e2[i * n], e1[i * n]), e = max(max(ep, eb), fx_em(fx_hi(h)) + 1);
-          out(o + i * sd, fx_to((a >> min(e - ep, 63)) + (R >> min(e - eb, 63)) + fx_from(h, e - 1), e));
+          const int eh = fx_em(fx_hi(h)) + 1;
+          int e;
+          long long r = fx_sum(a, max(e2[i * n], e1[i * n]), R, eb, e);
+          r = fx_sum(r, e, fx_from(h, eh - 1), eh, e);
+          out(o + i * sd, fx_to(r, e));
         }
       }
       if (l > 0) es[(l == 2 ? 0 : 5 * n2) + v * n2 + id] = eb;

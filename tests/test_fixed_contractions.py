@@ -187,3 +187,20 @@ def test_extreme_values(fx, n, etype, value):  # noqa: F811
             for stage in (0, 1):
                 fx.t_lift_modal(n, etype, ptr(H), ptr(F), 1, stage, ptr(R))
                 check(R, both)
+
+
+@pytest.mark.parametrize("n", [3, 5, 6])
+def test_derivative_sum_does_not_lean(fx, n):  # noqa: F811
+    """The mean error of many results, of lines on different exponents, is a small part of a single one's: errors that
+    lean one way add up in the integral behind (about 2 units of 2^-53 each at n = 6; 0.1 is five deviations of the mean)."""
+    rng = np.random.default_rng(n)
+    D = nodes(n)[1]
+    err = []
+    for _ in range(60):
+        G = rng.uniform(0.3, 1, (3, 5, n, n, n)) * 2.0 ** rng.uniform(-4, 0, (3, 5, 1, 1, 1)) * rng.choice([-1, 1], (3, 5, 1, 1, 1))
+        out, ref = np.empty((5, n, n, n)), np.zeros((5, n, n, n), LD)
+        fx.t_dsum(n, ptr(G), 7, ptr(out))
+        for l in range(3):
+            ref += np.moveaxis((along(G[l], l)[..., None].astype(LD) * D).sum(-2), -1, 1 + l)
+        err.append(out - ref)
+    assert abs(np.concatenate(err).mean()) < 0.1 * U
