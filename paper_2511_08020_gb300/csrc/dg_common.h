@@ -48,7 +48,8 @@ struct TypeTab {
   int W;        // [nQ]                   w_q (Gauss-Legendre weights times the Duffy Jacobian)
   int wA;       // [nQ][3][3]             w_q d(a,b,c)_l / d(xi,eta,zeta)_k
   int minv;     // [nM]                   1 / (V^T W V)_ii   (the mass matrix is diagonal)
-  int sqw;      // hexahedron: [nQ] sqrt(w_q), then [nQ] 1 / sqrt(w_q) (scaled nodal storage); -1 otherwise
+  int sqw;      // hexahedron: [nQ] sqrt(w_q), [nQ] 1 / sqrt(w_q) (scaled nodal storage), [nQ] w_q / sqrt(w_q) of
+                //   the exact weight (back to modal coefficients); -1 otherwise
   int fw;       // [nfaces][n*n]          reference face weights at the face points
   int sbp;      // hexahedron: [n][n] S_ij = w_i D_ij - w_j D_ji (D_ij = l'_j(x_i)), the antisymmetric
                 //   part of the 1D collocation operator W D (split form); -1 otherwise

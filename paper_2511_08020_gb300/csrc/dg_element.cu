@@ -814,9 +814,9 @@ __device__ __forceinline__ void process_element(const Ctx& c, int mode, const St
     return;
   }
   if constexpr (FAM == kMisc) if (mode == kScatter) {
-    // hexahedra only: storage s -> caller modal coefficients V^T W^{1/2} s
+    // hexahedra only: storage s -> caller modal coefficients V^{-1} W^{-1/2} s = V^T (w W^{-1/2}) s
     const double* S = io.Qin + qoff;
-    const double* sq = c.dpool + T.sqw;
+    const double* sq = c.dpool + T.sqw + 2 * nQ;
     for (int w = lane; w < 5 * nQ; w += blockDim.x) bufA[w] = S[w] * sq[w % nQ];
     __syncthreads();
     Epilogue ep{Epilogue::kStore, false, 1.0, io.Qout + c.elem_qoff[c.elem_of_slot[s]], nullptr, nullptr, nullptr,

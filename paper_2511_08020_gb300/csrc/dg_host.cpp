@@ -62,6 +62,24 @@ void gauss_legendre(int n, double* x, double* w) {
   if (n % 2 == 1) x[n / 2] = 0.0;
 }
 
+// Gauss-Legendre weights in extended precision from the nodes in double.
+static void gauss_weights(int n, const double* x, long double* w) {
+  for (int i = 0; i < n; ++i) {
+    long double z = x[i], dp = 1;
+    for (int it = 0; it < 4; ++it) {
+      long double p0 = 1, p1 = z;
+      for (int k = 2; k <= n; ++k) {
+        const long double p2 = ((2 * k - 1) * z * p1 - (k - 1) * p0) / k;
+        p0 = p1;
+        p1 = p2;
+      }
+      dp = n * (z * p1 - p0) / (z * z - 1);
+      if (it < 3) z -= p1 / dp;
+    }
+    w[i] = 2 / ((1 - z * z) * dp * dp);
+  }
+}
+
 // Jacobi P_n^(alpha,beta)(x) by the standard three-term recurrence.
 double jacobi(int n, double al, double be, double x) {
   if (n == 0) return 1.0;
@@ -419,6 +437,15 @@ int Tables::add(int type, int N, std::string* err) {
     t.sqw = (int)dpool.size();
     for (int q = 0; q < t.nQ; ++q) dput(std::sqrt(wq[q]));
     for (int q = 0; q < t.nQ; ++q) dput(1.0 / std::sqrt(wq[q]));
+    // w / sqrt(w_q) with w the weight in extended precision: V^T w V is the
+    // identity to rounding, where V^T W V of the doubles is up to 9e-16 off
+    // (the weights carry a few units of the last place per direction)
+    std::vector<long double> wl(n);
+    gauss_weights(n, x.data(), wl.data());
+    for (int i = 0; i < n; ++i)
+      for (int j = 0; j < n; ++j)
+        for (int k = 0; k < n; ++k)
+          dput((double)(wl[i] * wl[j] * wl[k] / dpool[t.sqw + (i * n + j) * n + k]));
   }
   // face descriptors + numerical check that the face rule points lie on the grid
   t.fw = (int)dpool.size();

@@ -119,6 +119,16 @@ void t_dense(int nM, const double* Md, const double* r, double* out) {
   });
 }
 void t_grad(int n, const double* U, double* out) { EACH(n, grad)(U, out); }
+// a hexahedron's modal coefficients to its storage and back, as dg_set_state and dg_get_state do
+int t_storage(int n, const double* Q, double* out) {
+  Setup s(HEX, n - 1);
+  const double* sq = s.c.dpool + s.T.sqw;
+  const int nQ = n * n * n;
+  double U[5 * 343];
+  EACH2(n, nodal, true)(HEX, Q, U, nullptr);
+  for (int o = 0; o < 5 * nQ; ++o) U[o] = U[o] * sq[o % nQ] * sq[2 * nQ + o % nQ];
+  return EACH2(n, modal, true)(HEX, U, out);
+}
 // nodes, Lagrange end values, and the factors of the basis at the nodes
 int t_tables(int n, int type, double* A, double* V, double* ext, int* face) {
   Setup s(type, n - 1);
