@@ -502,6 +502,32 @@ int Tables::add(int type, int N, std::string* err) {
     for (int r = 0; r < ipool[t.col_len + col]; ++r)
       ipool[t.mode_s + ipool[t.col_moff + col] + r] = balanced(t.C + ipool[t.col_coff + col] + r * n);
   for (int i = 0; i < 2 * n; ++i) fpool[t.ext + i] = split(dpool[t.ext + i], 3);   // kFxGE
+  // the kernels' 64-bit sums: sum (|h| |y| + l |x|) + 2^30 and sum |h| |x| + 2^32 of
+  // the operands h 2^31 + l, |h| <= 2^hb, 0 <= l < 2^31, over the `cnt` pairs at off
+  // with the given stride
+  auto fits = [&](int off, int cnt, int stride, int hb, double times = 1.0) {
+    double mid = 0.0, top = 0.0;
+    for (int k = 0; k < cnt; ++k) {
+      const double ax = std::fabs((double)fpool[off + k * stride].x), ay = std::fabs((double)fpool[off + k * stride].y);
+      mid += std::ldexp(ay, hb) + std::ldexp(ax, 31);
+      top += std::ldexp(ax, hb);
+    }
+    return times * mid + std::ldexp(1.0, 30) < std::ldexp(1.0, 63) && times * top + std::ldexp(1.0, 32) < std::ldexp(1.0, 63);
+  };
+  bool ok = true;
+  for (int p = 0; p < n; ++p) {
+    const int off = t.B + ipool[t.p_boff + p], len = ipool[t.p_blen + p];
+    for (int j = 0; j < n; ++j) ok = ok && fits(off + j, len, n, 30);
+    for (int r = 0; r < len; ++r) ok = ok && fits(off + r * n, n, 1, 30);
+  }
+  for (int col = 0; col < t.ncols; ++col) {
+    const int off = t.C + ipool[t.col_coff + col], len = ipool[t.col_len + col];
+    for (int k = 0; k < n; ++k) ok = ok && fits(off + k, len, n, 30);
+    for (int r = 0; r < len; ++r) ok = ok && fits(off + r * n, n, 1, 30);
+  }
+  // a node's six face values in one sum, or two of 62 bits
+  for (int i = 0; i < n; ++i) ok = ok && fits(t.ext + i, 2, n, 30, 3.0) && fits(t.ext + i, 2, n, 31);
+  if (!ok) { *err = "internal: integer tables out of range"; return -1; }
   for (int k = 0; k < 6; ++k) t.face_of[k] = -1;
   for (int lf = 0; lf < t.nfaces; ++lf) {
     const FaceDesc d = t.faces[lf];

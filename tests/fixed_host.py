@@ -129,6 +129,38 @@ int t_storage(int n, const double* Q, double* out) {
   for (int o = 0; o < 5 * nQ; ++o) U[o] = U[o] * sq[o % nQ] * sq[2 * nQ + o % nQ];
   return EACH2(n, modal, true)(HEX, U, out);
 }
+// largest 64-bit sum of the ragged passes and of the lift over its limit 2^63,
+// for operands h 2^31 + l with |h| <= 2^30 (2^31 in the lift at a node), 0 <= l < 2^31
+double t_bounds(int n, int type) {
+  Setup s(type, n - 1);
+  const TypeTab& T = s.T;
+  const int* ip = s.c.ipool;
+  double worst = 0.0;
+  auto sum = [&](int off, int cnt, int stride, int hb, double times) {
+    double mid = 0.0, top = 0.0;
+    for (int k = 0; k < cnt; ++k) {
+      const dgk::FixPair c = s.tb.fpool[off + k * stride];
+      mid += ldexp(fabs((double)c.y), hb) + ldexp(fabs((double)c.x), 31);
+      top += ldexp(fabs((double)c.x), hb);
+    }
+    worst = fmax(worst, ldexp(fmax(times * mid + ldexp(1.0, 30), times * top + ldexp(1.0, 32)), -63));
+  };
+  for (int p = 0; p < n; ++p) {
+    const int off = T.B + ip[T.p_boff + p], len = ip[T.p_blen + p];
+    for (int k = 0; k < n; ++k) sum(off + k, len, n, 30, 1.0);
+    for (int r = 0; r < len; ++r) sum(off + r * n, n, 1, 30, 1.0);
+  }
+  for (int col = 0; col < T.ncols; ++col) {
+    const int off = T.C + ip[T.col_coff + col], len = ip[T.col_len + col];
+    for (int k = 0; k < n; ++k) sum(off + k, len, n, 30, 1.0);
+    for (int r = 0; r < len; ++r) sum(off + r * n, n, 1, 30, 1.0);
+  }
+  for (int i = 0; i < n; ++i) {
+    sum(T.ext + i, 2, n, 30, 3.0);
+    sum(T.ext + i, 2, n, 31, 1.0);
+  }
+  return worst;
+}
 // nodes, Lagrange end values, and the factors of the basis at the nodes
 int t_tables(int n, int type, double* A, double* V, double* ext, int* face) {
   Setup s(type, n - 1);
