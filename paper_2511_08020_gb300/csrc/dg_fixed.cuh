@@ -286,11 +286,9 @@ __device__ __forceinline__ unsigned fx_mag(long long R) {
   return (unsigned)(h ^ (h >> 31));
 }
 
-// a b + c: one IMAD.WIDE as long as the compiler cannot prove the sign of an
-// operand (it then forms a 64-bit product of three instructions; fx_split hides
-// the sign of l).  mad.wide.s32 written as inline PTX is no help: half of its
-// additions become separate instructions (158 against 109 per five dot
-// products of five terms).
+// a b + c, 32 x 32 + 64 bits.  The low words pass through an empty asm statement
+// (fx_split), so that the compiler does not know their sign: two steps of the
+// mixed 16^3 mesh at N = 4 take 5.33 ms, 5.67 without (viscous 20^3 18.1, 19.1).
 __device__ __forceinline__ long long fx_madw(int a, int b, long long c) { return (long long)a * b + c; }
 
 __device__ __forceinline__ unsigned fx_hi(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }

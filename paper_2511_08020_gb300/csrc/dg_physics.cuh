@@ -26,8 +26,8 @@ __device__ __forceinline__ unsigned smid() {
 // 1/a: the hardware's estimate x (20 bits or more) and one step of
 // Householder's method of order two, x + x (e + e^2) with e = 1 - a x; the
 // neglected e^3 is below 2^-60, so the result is the rounded quotient but for
-// a few parts in 2^7 of the last bit.  Five FP64 instructions instead of the
-// division's ten.  Arguments near the ends of the range take the division.
+// a few parts in 2^7 of the last bit (0.51 units of it at most, the division
+// 0.5).  Arguments near the ends of the range take the division.
 __device__ __forceinline__ double rcp(double a) {
   const unsigned ex = ((unsigned)__double2hiint(a) >> 20) & 0x7ffu;
   if (ex - 30u > 1980u) return 1.0 / a;
@@ -80,10 +80,9 @@ __device__ __forceinline__ void normal_state(const double* U, const double* n, d
 //   lam       = max(|us-| + (wS/2) c-, |us+| + (wS/2) c+),
 // one reciprocal and one square root per side.  fmax passes over the NaN of a
 // side whose pressure is negative, so the other side's speed is taken there.
-// The face kernel is bound by FP64 issue: about 75 instructions per point, 105
-// with IEEE division, root and separate side fluxes (16^3 mixed N = 4: 151 us,
-// 140 with the reciprocals alone, 130 in this form; the Navier-Stokes flux phase
-// at 12^3 164 -> 128 us).
+// The face kernel is bound by FP64 issue (16^3 mixed N = 4: 151 us with the
+// division, the root and separate side fluxes, 140 with the reciprocals alone,
+// 130 in this form; the Navier-Stokes flux phase at 12^3 164 -> 128 us).
 struct LfSide {
   double r, p, ms, us, lam;
 };
@@ -349,8 +348,8 @@ __device__ __forceinline__ void viscous_flux(const double* W, const double* g, d
 
 // Viscous flux through a face, F_v.s for a (scaled) normal s, from 1/rho, the
 // velocity, p and the gradient: q[0..2] momentum, q[3] energy.  The traction is
-// contracted with s before the stress is formed (41 FP64 instructions; the
-// three fluxes and their contraction took about 75).
+// contracted with s before the stress is formed: about half the operations of
+// the three fluxes and their contraction.
 __device__ __forceinline__ void viscous_flux_normal(double r, const double* u, double p, const double* g,
                                                     const double* s, double mu, double kappa, double* q) {
   const double lam = (2.0 / 3.0) * mu * (g[1] + g[5 + 2] + g[10 + 3]);
