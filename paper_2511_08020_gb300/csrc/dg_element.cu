@@ -436,7 +436,7 @@ __device__ __forceinline__ void element_forward_split(const Ctx& c, const TypeTa
 template <bool ANY>
 __device__ __forceinline__ void element_forward_t(const Ctx& c, const TypeTab& T, int64_t s, double* bufA, double* bufG,
                                                   int lane) {
-  constexpr int n = kn, nQ = knQ, n2 = kn2;
+  constexpr int nQ = knQ;
   const double* dp = c.dpool;
   if (T.type == HEX) {
     modal_to_nodal(c, T, bufG, bufA, bufG, lane);
@@ -611,7 +611,7 @@ __device__ __forceinline__ void lift_scaled_t(const Ctx& c, const TypeTab& T, in
 // their own: fewer resident blocks, and the phase waits for latencies).
 template <bool CURVED>
 __device__ __forceinline__ void element_ns_volume_t(const Ctx& c, const TypeTab& T, int64_t s, double* smem, int lane) {
-  constexpr int n = kn, nQ = knQ, n2 = kn2;
+  constexpr int nQ = knQ, n2 = kn2;
   // curved element: pointwise metric [9][nQ], J, 1/J, (prism, pyramid) dense M_e^{-1}
   const double* cblk = CURVED ? c.cpool + c.slot_coff[s] : nullptr;
   constexpr int nQm = knQ;
@@ -947,7 +947,7 @@ __device__ __forceinline__ void element_vjp_a_t(const Ctx& c, const VjpArgs& va,
   // (prism, pyramid) in place of the affine 1/J and diagonal M_ref^{-1}
   const double* cblk = CURVED ? c.cpool + c.slot_coff[s] : nullptr;
   const bool dense = CURVED && T.type != HEX;
-  constexpr int n = kn, nQ = knQ, n2 = kn2;
+  constexpr int nQ = knQ;
   const int nM = T.nM;
   const double* dp = c.dpool;
   const int64_t qoff = c.slot_qoff[s];
@@ -1081,7 +1081,7 @@ __device__ __forceinline__ void lift_add(const Ctx& c, const TypeTab& T, int64_t
 template <bool CURVED>
 __device__ __forceinline__ void element_vjp_a_ns_t(const Ctx& c, const VjpArgs& va, int64_t s, double* smem, int lane) {
   const TypeTab& T = c.tabs[c.slot_tab[s]];
-  constexpr int n = kn, nQ = knQ, n2 = kn2;
+  constexpr int nQ = knQ;
   const int nM = T.nM;
   constexpr int nQm = knQ;
   double* bufY = smem;
@@ -1192,7 +1192,7 @@ template <bool CURVED>
 __device__ __forceinline__ void element_vjp_b_ns_t(const Ctx& c, int64_t s, double* smem, int lane) {
   const TypeTab& T = c.tabs[c.slot_tab[s]];
   const double* cblk = CURVED ? c.cpool + c.slot_coff[s] : nullptr;
-  constexpr int n = kn, nQ = knQ, n2 = kn2;
+  constexpr int nQ = knQ, n2 = kn2;
   const int nf = T.nfaces;
   constexpr int nQm = knQ;
   double* bufD = smem;                 // smem + 15 nQm .. 20 nQm is scratch
@@ -1658,7 +1658,7 @@ __global__ void __launch_bounds__(kMassThreads, MINB) moving_mass_kernel(Ctx c, 
     const int64_t s = list[e];
     const TypeTab& T = c.tabs[c.slot_tab[s]];
     constexpr int nQ = knQ;
-  const int nM = T.nM;
+    const int nM = T.nM;
     const int64_t qoff = c.slot_qoff[s];
     const double* m = c.mpool + c.slot_moff[s];
     if (T.type == HEX) {

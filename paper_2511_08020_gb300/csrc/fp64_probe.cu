@@ -1,6 +1,6 @@
-// FP64 throughput probes for the benchmark's roofline denominators (not part
-// of libdg.so): a DFMA-chain loop, an mma.sync f64 m8n8k4 loop, and both at
-// once in one launch.  Built into _lib/libfp64probe.so; bench.py loads it.
+// Throughput probes for the benchmark's roofline denominators (not part of
+// libdg.so): a DFMA-chain loop, an mma.sync f64 m8n8k4 loop, both at once in one
+// launch, and a loop of 32 x 32 + 64 bit integer multiply-adds.  Built into _lib/libfp64probe.so; bench.py loads it.
 #include <cuda_runtime.h>
 
 namespace {
@@ -33,6 +33,21 @@ __global__ void dmma_probe_kernel(double* out, int iters) {
   double t = 0;
   for (int k = 0; k < 4; ++k) t += c0[k] + c1[k];
   out[blockIdx.x * blockDim.x + threadIdx.x] = t;
+}
+
+// Chains of integer multiply-adds, 32 x 32 + 64 bits.
+__global__ void int_mad_probe_kernel(double* out, int iters, unsigned s) {
+  unsigned long long a[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) a[k] = threadIdx.x + 77u * k + 1u;
+  for (int i = 0; i < iters; ++i) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) a[k] = (unsigned long long)(unsigned)a[k] * s + a[k];
+  }
+  unsigned long long t = 0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) t += a[k];
+  out[blockIdx.x * blockDim.x + threadIdx.x] = (double)t;
 }
 
 // Half the warps of a block run DFMA chains, the other half mma.sync f64:
@@ -132,6 +147,34 @@ static cudaError_t probe_mixed(double* total_tflops) {
   return e;
 }
 
+static cudaError_t probe_int_mad(double* tmads) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int blocks = sms * 8, threads = 256, it = 40000;
+  double* out = nullptr;
+  e = cudaMalloc(&out, sizeof(double) * blocks * threads);
+  if (e != cudaSuccess) return e;
+  cudaEvent_t e0, e1;
+  cudaEventCreate(&e0);
+  cudaEventCreate(&e1);
+  int_mad_probe_kernel<<<blocks, threads>>>(out, 10, 2654435761u);
+  cudaEventRecord(e0);
+  int_mad_probe_kernel<<<blocks, threads>>>(out, it, 2654435761u);
+  cudaEventRecord(e1);
+  cudaEventSynchronize(e1);
+  float ms = 0.f;
+  cudaEventElapsedTime(&ms, e0, e1);
+  *tmads = 8.0 * it * (double)blocks * threads / (ms * 1e-3) / 1e12;
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  e = cudaGetLastError();
+  cudaFree(out);
+  return e;
+}
+
 extern "C" {
 
 // Measured FP64 throughput of the current device (DFMA chains and mma.sync f64
@@ -148,6 +191,13 @@ int fp64_probe_peak(double* dfma_tflops, double* dmma_tflops) {
 int fp64_probe_mixed(double* total_tflops) {
   if (!total_tflops) return (int)cudaErrorInvalidValue;
   return (int)probe_mixed(total_tflops);
+}
+
+// Measured rate of 32 x 32 + 64 bit integer multiply-adds, 1e12 per second, of a
+// ~50 ms probe launch.  Synchronises.
+int int_mad_probe(double* tmads) {
+  if (!tmads) return (int)cudaErrorInvalidValue;
+  return (int)probe_int_mad(tmads);
 }
 
 }  // extern "C"
