@@ -1,7 +1,7 @@
 // Fixed-point contractions of the element kernels.
 //
 // FP64 issues 2 DFMA per clock and SM on this part (measured 1.71), the
-// 32 x 32 + 64 bit integer multiply-add 64 (measured 61).  A dot product of n
+// 32 x 32 + 64 bit integer multiply-add 64 (measured 63).  A dot product of n
 // doubles with table coefficients is therefore done on integers: the n values
 // share one exponent (their largest), become 61-bit integers D = dh 2^31 + dl,
 // the coefficients are 62-bit integers C = ch 2^31 + cl, and

@@ -36,15 +36,16 @@ __global__ void dmma_probe_kernel(double* out, int iters) {
 }
 
 // Chains of integer multiply-adds, 32 x 32 + 64 bits.
-__global__ void int_mad_probe_kernel(double* out, int iters, unsigned s) {
-  unsigned long long a[8];
+__global__ void int_mad_probe_kernel(double* out, int iters, int s) {
+  long long a[8];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) a[k] = threadIdx.x + 77u * k + 1u;
+  for (int k = 0; k < 8; ++k) a[k] = threadIdx.x + 77 * k + 1;
+  const int x = threadIdx.x * 3 + 1;
   for (int i = 0; i < iters; ++i) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) a[k] = (unsigned long long)(unsigned)a[k] * s + a[k];
+    for (int k = 0; k < 8; ++k) asm volatile("mad.wide.s32 %0, %1, %2, %0;" : "+l"(a[k]) : "r"(x), "r"(s));
   }
-  unsigned long long t = 0;
+  long long t = 0;
 #pragma unroll
   for (int k = 0; k < 8; ++k) t += a[k];
   out[blockIdx.x * blockDim.x + threadIdx.x] = (double)t;
@@ -153,16 +154,16 @@ static cudaError_t probe_int_mad(double* tmads) {
   if (e != cudaSuccess) return e;
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int blocks = sms * 8, threads = 256, it = 40000;
+  const int blocks = sms * 8, threads = 256, it = 80000;
   double* out = nullptr;
   e = cudaMalloc(&out, sizeof(double) * blocks * threads);
   if (e != cudaSuccess) return e;
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  int_mad_probe_kernel<<<blocks, threads>>>(out, 10, 2654435761u);
+  int_mad_probe_kernel<<<blocks, threads>>>(out, 10, 3);
   cudaEventRecord(e0);
-  int_mad_probe_kernel<<<blocks, threads>>>(out, it, 2654435761u);
+  int_mad_probe_kernel<<<blocks, threads>>>(out, it, 3);
   cudaEventRecord(e1);
   cudaEventSynchronize(e1);
   float ms = 0.f;
@@ -194,7 +195,7 @@ int fp64_probe_mixed(double* total_tflops) {
 }
 
 // Measured rate of 32 x 32 + 64 bit integer multiply-adds, 1e12 per second, of a
-// ~50 ms probe launch.  Synchronises.
+// ~10 ms probe launch.  Synchronises.
 int int_mad_probe(double* tmads) {
   if (!tmads) return (int)cudaErrorInvalidValue;
   return (int)probe_int_mad(tmads);
