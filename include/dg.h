@@ -358,7 +358,7 @@ dg_status dg_mesh_layout(const dg_mesh* mesh, int64_t* n_dof, int64_t* slot_of_e
 
 /* Convert a state (or a cotangent) between the caller layout Q_ext and the
  * storage layout: element blocks permuted, hexahedra's modal coefficients Q
- * mapped to W^{1/2} V Q and back by V^T W^{1/2}.  Q_ext and Q_store must not
+ * mapped to W^{1/2} V Q and back by its inverse.  Q_ext and Q_store must not
  * overlap.  is_device = 1: Q_ext is a device pointer and the call is asynchronous;
  * is_device = 0: Q_ext is host memory (pinned or pageable) and the call
  * synchronises `stream` before returning. */
